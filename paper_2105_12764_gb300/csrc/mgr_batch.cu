@@ -14,13 +14,12 @@
 // stream order inside the graph, so no CTA ever waits on another.
 //
 // Autotuning (Sec. III.B: an analytic model ranks the candidate launch
-// shapes, the best few are measured): candidates are the level-pass tile
-// (8 warps x 2 row pairs = 30x14 coarse nodes, 4 warps x 2 = 30x6, or 4 warps
-// in half-warp row groups x 2 = 14x14, for fields whose coarse rows are
-// short) and the z-chunk length (at most 8, 16 or 32 coarse planes, split evenly over a
-// field's items).  The model charges each work item the shared-memory slots
-// it streams (halo and padding included) and takes the longer of the memory
-// time and the longest-processing-time schedule of the items over the
+// shapes, the best few are measured): candidates are the level pass's strips
+// (14 or 6 coarse rows in whole-warp row groups, 14 in half-warp ones; rows are
+// split evenly over a field's strips) and the z-chunk length (at most 8, 16 or 32
+// coarse planes, split evenly over a field's items).  The model charges each work
+// item the slots it streams (halo and padding included) and takes the longer of
+// the memory time and the longest-processing-time schedule of the items over the
 // persistent CTAs; the model's best candidate of each tile shape, the next
 // best up to three, and the other chunk lengths of the fastest tile shape are
 // timed on the real batch and the fastest is cached per batch shape.
@@ -38,6 +37,7 @@
 #include <queue>
 #include <string>
 #include <thread>
+#include <type_traits>
 #include <vector>
 
 #include "mgr_internal.h"
@@ -62,17 +62,18 @@ __device__ __forceinline__ void copy_words(T* dst, const T* src) {
   for (int i = threadIdx.x; i < int(sizeof(T) / 4); i += blockDim.x) d[i] = s[i];
 }
 
-template <int MODE, int NW, int RPW, int STAGES, typename TI, typename TD, typename TS, typename TW, int LX = 32>
-__global__ void __launch_bounds__(NW * 32, level_ctas_per_sm(NW)) kb_level(const LevelArgs<TS, TW>* __restrict__ args,
+// One warp per CTA: a level-pass item is one warp's strip columns and z chunk.
+template <int MODE, typename TI, typename TD, typename TS, typename TW, bool S1, int LX = 32>
+__global__ void __launch_bounds__(32, level_ctas<MODE, TS>()) kb_level(const LevelArgs<TS, TW>* __restrict__ args,
                                                        const int4* __restrict__ items, int n) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(16) LevelArgs<TS, TW> sa;
   for (int i = blockIdx.x; i < n; i += gridDim.x) {
     const int4 it = items[i];
     copy_words(&sa, args + it.x);
-    __syncthreads();
-    level_body<MODE, NW, RPW, STAGES, TI, TD, TS, TW, false, false, false, LX>(sa, it.y, it.z, it.w, smem_raw);
-    __syncthreads();
+    __syncwarp();
+    level_body<MODE, TI, TD, TS, TW, S1, false, false, false, LX>(sa, it.y, it.w, smem_raw);
+    __syncwarp();
   }
 }
 
@@ -209,30 +210,32 @@ struct FieldRef {
   char* ws;
 };
 
-// Level-pass tile candidates (NW warps x RPW row pairs per row group of LX
-// lanes); chunk lengths.
+// Level-pass tile candidates (coarse rows per strip, lanes per row group);
+// chunk lengths.
 struct TileCand {
-  int cfg;    // 0: 8 warps x 2 row pairs (30 x 14), 1: 4 warps x 2 (30 x 6),
-              // 2: 4 warps as 8 half-warp row groups x 2 (14 x 14)
+  int cfg;    // 0: strips of 14 coarse rows, 1: of 6, both in whole-warp row groups (30 outputs);
+              // 2: 14 rows in half-warp row groups (14 outputs)
   int chunk;  // coarse z planes per work item
 };
 constexpr int kNumCfg = 3;
-inline int cfg_bx(int cfg) { return cfg == 2 ? 14 : 30; }
+inline int cfg_lanes(int cfg) { return cfg == 2 ? 16 : 32; }
 inline int cfg_by(int cfg) { return cfg == 1 ? 6 : 14; }
 inline const char* cfg_name(int cfg) { return cfg == 0 ? "30x14" : cfg == 1 ? "30x6" : "14x14"; }
-
-inline int ctas_per_sm(int cfg) { return cfg == 0 ? 2 : 4; }
 
 // z-chunk length candidates of the autotuner (coarse planes per work item, at most)
 #ifndef MGR_BATCH_CHUNK_MAX
 #define MGR_BATCH_CHUNK_MAX 32
 #endif
-static_assert(MGR_BATCH_CHUNK_MAX <= kLevelMaxChunk, "level-pass chunks are at most kLevelMaxChunk planes");
+static_assert(MGR_BATCH_CHUNK_MAX <= kLevelMaxChunk, "interpolation chunks are at most kLevelMaxChunk planes");
 #if MGR_BATCH_CHUNK_MAX > 32
 constexpr int kChunks[] = {8, 16, 32, MGR_BATCH_CHUNK_MAX};
 #else
 constexpr int kChunks[] = {8, 16, 32};
 #endif
+
+// Resident one-warp level-pass CTAs per SM a persistent launch asks for (the
+// shared memory of 14-row strips allows 18 in FP32).
+constexpr int kLevelResident = 16;
 
 // Coarse z planes per work item: at most `chunk`, split evenly over the items
 // (33 planes in chunks of 32 are 17 + 16, not 32 + 1).
@@ -301,16 +304,21 @@ struct Builder {
       a.m[k] = g.ax[k].m;
       a.s[k] = g.ax[k].s;
       a.N[k] = g.ax[k].N;
-      a.wa[k] = T + g.ax[k].o_wa;
-      a.wb[k] = T + g.ax[k].o_wb;
-      a.k[k] = T + g.ax[k].o_k;
+      a.slot[k] = T + g.ax[k].o_slot;
     }
     a.y_sz = p->full[1] * p->full[2];
     a.y_sy = p->full[2];
     a.c_sz = int64_t(g.ax[1].m) * g.ax[2].m;
     a.c_sy = g.ax[2].m;
+    a.rows = balanced_chunk(cfg_by(cand.cfg), g.ax[1].m);
     a.qz_chunk = balanced_chunk(cand.chunk, g.ax[0].m);
     return a;
+  }
+
+  // Warps over the strips of a level's xy grid.
+  int64_t warps_of(int mx, int my) const {
+    const int r = balanced_chunk(cfg_by(cand.cfg), my);
+    return cfg_lanes(cand.cfg) == 32 ? level_warps<32>(mx, my, r) : level_warps<16>(mx, my, r);
   }
 
   // Level-pass phase for all fields at depth d.
@@ -318,7 +326,7 @@ struct Builder {
   void level_phase(int d, bool first_dec) {
     std::vector<LevelArgs<TS, TW>> descs;
     std::vector<int4> items;
-    const int BX = cfg_bx(cand.cfg), BY = cfg_by(cand.cfg);
+    size_t smem = 0;  // the largest item's
     for (size_t fi = 0; fi < fields.size(); ++fi) {
       const FieldRef& fr = fields[fi];
       const int L = fr.p->levels;
@@ -334,19 +342,16 @@ struct Builder {
         a.write_y = 1;
         if (l == L) {
           a.in = fr.in;
-          a.in_full = 1;
           a.in_sz = a.y_sz;
           a.in_sy = a.y_sy;
         } else {
           const LevelGeom& g = fr.p->geom[l];
           a.in = cur;
-          a.in_full = 0;
           a.in_sz = int64_t(g.ax[1].n) * g.ax[2].n;
           a.in_sy = g.ax[2].n;
         }
       } else {
         a.in = fr.in;
-        a.in_full = 1;
         a.in_sz = a.y_sz;
         a.in_sy = a.y_sy;
         a.f = reinterpret_cast<TW*>(bufF(fr));
@@ -356,10 +361,10 @@ struct Builder {
       }
       const int di = int(descs.size());
       descs.push_back(a);
-      const int gx = (a.m[2] + BX - 1) / BX, gy = (a.m[1] + BY - 1) / BY, gz = (a.m[0] + a.qz_chunk - 1) / a.qz_chunk;
+      smem = std::max(smem, level_smem_bytes<MODE, TI, TS>(a.rows, level_slot_rows(a.m[2], a.m[1], a.rows)));
+      const int gx = int(warps_of(a.m[2], a.m[1])), gz = (a.m[0] + a.qz_chunk - 1) / a.qz_chunk;
       for (int z = 0; z < gz; ++z)
-        for (int y = 0; y < gy; ++y)
-          for (int x = 0; x < gx; ++x) items.push_back(make_int4(di, x, y, z));
+        for (int x = 0; x < gx; ++x) items.push_back(make_int4(di, x, 0, z));
     }
     (void)first_dec;
     if (items.empty()) return;
@@ -368,23 +373,16 @@ struct Builder {
     ph.desc_off = blob.put(descs.data(), descs.size() * sizeof(descs[0]));
     ph.items_off = blob.put(items.data(), items.size() * sizeof(int4));
     ph.n_items = int(items.size());
-    if (cand.cfg == 0) {
-      using C = LevelCfg<TS>;
-      ph.fn = reinterpret_cast<const void*>(kb_level<MODE, C::NW, C::RPW, C::STAGES, TI, TD, TS, TW>);
-      ph.block = C::NW * 32;
-      ph.smem = level_smem_bytes<C::NW, C::RPW, C::STAGES, TI, TS>();
-    } else if (cand.cfg == 1) {
-      constexpr int ST = LevelCfg<TS>::STAGES;
-      ph.fn = reinterpret_cast<const void*>(kb_level<MODE, 4, 2, ST, TI, TD, TS, TW>);
-      ph.block = 128;
-      ph.smem = level_smem_bytes<4, 2, ST, TI, TS>();
-    } else {
-      constexpr int ST = LevelCfg<TS>::STAGES;
-      ph.fn = reinterpret_cast<const void*>(kb_level<MODE, 4, 2, ST, TI, TD, TS, TW, 16>);
-      ph.block = 128;
-      ph.smem = level_smem_bytes<4, 2, ST, TI, TS, 16>();
-    }
-    ph.grid = std::min(ph.n_items, num_sms * ctas_per_sm(cand.cfg));
+    const bool wide = cfg_lanes(cand.cfg) == 32;
+    if (d == 0)  // the finest level: unit stride
+      ph.fn = wide ? reinterpret_cast<const void*>(kb_level<MODE, TI, TD, TS, TW, true>)
+                   : reinterpret_cast<const void*>(kb_level<MODE, TI, TD, TS, TW, true, 16>);
+    else
+      ph.fn = wide ? reinterpret_cast<const void*>(kb_level<MODE, TI, TD, TS, TW, false>)
+                   : reinterpret_cast<const void*>(kb_level<MODE, TI, TD, TS, TW, false, 16>);
+    ph.block = 32;
+    ph.smem = smem;
+    ph.grid = std::min(ph.n_items, num_sms * kLevelResident);
     pending.push_back(ph);
   }
 
@@ -670,15 +668,14 @@ struct Builder {
   }
 
   // Estimated time of this candidate (model of Sec. III.B, restated): every
-  // level-pass item streams RR x RC slots per plane pair (halo and padding
-  // included); the phase takes the longer of that traffic at HBM speed and
-  // the LPT schedule of the items over the persistent CTAs.
+  // level-pass item streams (2 rows + 3) x 64 slots per plane pair (halo and
+  // padding included); the phase takes the longer of that traffic at HBM speed
+  // and the LPT schedule of the items over the persistent CTAs.
   double model_cost(double hbm_bytes_per_us) const {
     double total = 0;
-    const int BX = cfg_bx(cand.cfg), BY = cfg_by(cand.cfg);
-    const int RR = 2 * (BY + 2), RC = 2 * (BX + 2);
-    const int slots = num_sms * ctas_per_sm(cand.cfg);
-    const double t_iter_us = (cand.cfg == 0 ? 1.6 : 1.0);
+    const int slots = num_sms * kLevelResident;
+    // one warp's time per unit (a row pair of a plane pair), most of the resident warps busy
+    const double t_unit_us = sizeof(TS) == 8 ? 4.0 : 0.7;
     int D = 0;
     for (const FieldRef& fr : fields) D = std::max(D, fr.p->levels);
     for (int d = 0; d < D; ++d) {
@@ -690,13 +687,14 @@ struct Builder {
         if (!tiled(fi, d)) continue;
         const LevelGeom& g = fr.p->geom[L - d];
         const int chunk = balanced_chunk(cand.chunk, g.ax[0].m);
-        const int gx = (g.ax[2].m + BX - 1) / BX, gy = (g.ax[1].m + BY - 1) / BY;
+        const int rows = balanced_chunk(cfg_by(cand.cfg), g.ax[1].m);
+        const int64_t gx = warps_of(g.ax[2].m, g.ax[1].m);
         const int gz = (g.ax[0].m + chunk - 1) / chunk;
         for (int z = 0; z < gz; ++z) {
           const int planes = std::min(chunk, g.ax[0].m - z * chunk) + 1;
-          for (int i = 0; i < gx * gy; ++i) {
-            jobs.push_back(planes * t_iter_us + 2.0);
-            bytes += double(planes) * 2.0 * RR * RC * fr.p->elem;
+          for (int64_t i = 0; i < gx; ++i) {
+            jobs.push_back(planes * (rows + 2) * t_unit_us + 2.0);
+            bytes += double(planes) * 2.0 * (2 * rows + 3) * 64 * fr.p->elem;
           }
         }
       }

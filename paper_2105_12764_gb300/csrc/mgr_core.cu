@@ -4,16 +4,15 @@
 // One decomposition level l (n nodes -> m coarse nodes) is three kinds of
 // launches (the paper's GPK / LPK / IPK roles, redesigned):
 //
-//   k_level_load   coefficients (Sec. II.A.1) and the load vector
+//   k_level        coefficients (Sec. II.A.1) and the load vector
 //                  f' = (x_k D_k^-1 P_k^T M_k) c (Sec. II.A.2, III.A.2) in one
-//                  pass.  A CTA owns a (BY x BX) tile of coarse (y, x) nodes and
-//                  a chunk of coarse z planes; it streams the fine z planes of
-//                  its tile region (with a two-node halo for the 5-tap stencil)
-//                  through shared memory with cp.async double buffering,
-//                  computes the coefficients of each plane, writes them to the
-//                  nodal output, applies the x and y stencils in shared memory
-//                  and accumulates the z stencil in registers.  The coarse nodal
-//                  values go to a compact coarse workspace.
+//                  pass.  A warp owns a strip of coarse y rows for the coarse x
+//                  nodes of its lanes and a chunk of coarse z planes; it streams the
+//                  fine z planes of its region, forms the coefficients of each,
+//                  writes them to the nodal output, applies the x stencil by
+//                  shuffles, the y stencil in registers and accumulates the z
+//                  stencil.  The coarse nodal values go to a compact coarse
+//                  workspace.
 //   k_solve_*      the Thomas recurrences along one axis of the compact coarse
 //                  grid (Sec. III.A.3).  Strided axes: one thread per line,
 //                  coalesced across the contiguous axis.  The contiguous axis:
@@ -170,6 +169,8 @@ cudaError_t coarsest_q_launch(const mgr_plan* p, int* codes, TV* v, double q, in
 // The finest level pass of a pipelined host-buffer decomposition: part k
 // covers the pass's z chunks [c0[k], c0[k+1]), waits for wait[k] (its input
 // planes are on the device) and records done[k].
+// The pass's shape is chosen for the planes of one part.
+inline int pipe_planes(int mz) { return (mz + kPipeParts - 1) / kPipeParts; }
 struct PipeParts {
   int parts;
   const int* c0;
@@ -227,13 +228,12 @@ cudaError_t decompose_t(const mgr_plan* p, const void* in, void* out, void* ws, 
     rec_begin(st);
     if (l == L) {
       a.in = in;
-      a.in_full = 1;
       a.in_sz = p->full[1] * p->full[2];
       a.in_sy = p->full[2];
       if (pp) {
         for (int k = 0; k < pp->parts; ++k) {
           if (cudaStreamWaitEvent(st, pp->wait[k], 0) != cudaSuccess) return cudaGetLastError();
-          launch_level_chunks<0, TD, TY, TS, TW, PK, QZ>(p, a, pp->c0[k], pp->c0[k + 1], st);
+          launch_level_chunks<0, TD, TY, TS, TW, PK, QZ>(p, a, pp->c0[k], pp->c0[k + 1], st, pipe_planes(g.ax[0].m));
           if (cudaEventRecord(pp->done[k], st) != cudaSuccess) return cudaGetLastError();
         }
       } else {
@@ -241,7 +241,6 @@ cudaError_t decompose_t(const mgr_plan* p, const void* in, void* out, void* ws, 
       }
     } else {
       a.in = cur;
-      a.in_full = 0;
       a.in_sz = int64_t(g.ax[1].n) * g.ax[2].n;
       a.in_sy = g.ax[2].n;
       launch_level<0, TW, TY, TS, TW, PK, QZ>(p, a, st);
@@ -333,11 +332,9 @@ cudaError_t recompose_t(const mgr_plan* p, const void* in, void* out, void* ws, 
     auto a = level_args<TS, TW>(p, l);
     a.in = PK ? static_cast<const void*>(static_cast<const TY*>(in) + p->class_off[l]) : in;
     if (PK) {
-      a.in_full = 0;
       a.in_sz = int64_t(g.ax[1].n) * g.ax[2].n;
       a.in_sy = g.ax[2].n;
     } else {
-      a.in_full = 1;
       a.in_sz = a.y_sz;
       a.in_sy = a.y_sy;
     }
@@ -350,7 +347,7 @@ cudaError_t recompose_t(const mgr_plan* p, const void* in, void* out, void* ws, 
     if (rp && l == L) {
       for (int k = 0; k < rp->parts; ++k) {
         if (cudaStreamWaitEvent(s, rp->odd[k], 0) != cudaSuccess) return cudaGetLastError();
-        launch_level_chunks<1, TY, TY, TS, TW, PK, QZ>(p, a, rp->c0[k], rp->c0[k + 1], s);
+        launch_level_chunks<1, TY, TY, TS, TW, PK, QZ>(p, a, rp->c0[k], rp->c0[k + 1], s, pipe_planes(g.ax[0].m));
       }
     } else {
       launch_level<1, TY, TY, TS, TW, PK, QZ>(p, a, s);
@@ -468,8 +465,7 @@ cudaError_t host_pipe_t(const mgr_plan* p, const void* host_in, void* host_out, 
   const int nz = int(p->full[0]), mz = p->geom[L].ax[0].m;
   const size_t plane = size_t(p->full[1]) * size_t(p->full[2]) * sizeof(TD);
   auto a = level_args<TS, TW>(p, L);
-  const dim3 grid = level_grid<0>(p, a);
-  const int gz = int(grid.z), qc = a.qz_chunk;
+  const int gz = int(level_grid<0, TD, false>(p, a, pipe_planes(mz)).y), qc = a.qz_chunk;
   const int parts = std::min(gz, kPipeParts);
   int c0[kPipeParts + 1];
   for (int k = 0; k <= parts; ++k) c0[k] = int((int64_t(k) * gz) / parts);
@@ -535,7 +531,7 @@ cudaError_t host_rec_pipe_t(const mgr_plan* p, const void* host_in, void* host_o
   const int nz = int(p->full[0]), mz = p->geom[L].ax[0].m;
   const size_t plane = size_t(p->full[1]) * size_t(p->full[2]) * sizeof(TD);
   auto a = level_args<TS, TW>(p, L);
-  const int gz = int(level_grid<1>(p, a).z), qc = a.qz_chunk;
+  const int gz = int(level_grid<1, TD, false>(p, a, pipe_planes(mz)).y), qc = a.qz_chunk;
   const int parts = std::min(gz, kPipeParts);
   int c0[kPipeParts + 1];
   for (int k = 0; k <= parts; ++k) c0[k] = int((int64_t(k) * gz) / parts);

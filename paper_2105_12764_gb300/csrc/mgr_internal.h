@@ -24,6 +24,8 @@ namespace mgr {
 
 constexpr int kAxes = 3;
 constexpr int kMaxLevels = 60;
+// Slot table of an axis: entries per coarse node (see mgr_level.cuh)
+constexpr int kSlot = 8;
 
 // Element type combination of one plan ("form").
 enum Form : int {
@@ -44,6 +46,8 @@ struct AxisLevel {
   int64_t o_wa = 0, o_wb = 0;  // interpolation weights, indexed by fine node (n entries)
   int64_t o_k = 0;             // 5 * m mass-transfer taps, row q at offsets -2..2 around node min(2q, n-1),
                                // each row scaled by 1/u_q of the coarse mass matrix's LU factors
+  int64_t o_slot = 0;          // kSlot * m slot entries: per coarse node q its row's weights on the slots (q-1).own,
+                               // (q-1).fine, q.own, q.fine, (q+1).own, then q.fine's interpolation weights
   int64_t o_ta = 0, o_tb = 0;  // scaled Thomas recurrences, m entries each
 };
 

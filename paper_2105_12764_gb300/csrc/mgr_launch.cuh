@@ -65,9 +65,7 @@ LevelArgs<TS, TW> level_args(const mgr_plan* p, int l) {
     a.m[k] = g.ax[k].m;
     a.s[k] = g.ax[k].s;
     a.N[k] = g.ax[k].N;
-    a.wa[k] = T + g.ax[k].o_wa;
-    a.wb[k] = T + g.ax[k].o_wb;
-    a.k[k] = T + g.ax[k].o_k;
+    a.slot[k] = T + g.ax[k].o_slot;
   }
   a.y_sz = p->full[1] * p->full[2];
   a.y_sy = p->full[2];
@@ -100,42 +98,92 @@ inline int choose_chunks(const mgr_plan* p, int64_t tiles, int mz, int ctas_per_
   return best;
 }
 
-template <int MODE, typename TS, typename TW>
-dim3 level_grid(const mgr_plan* p, LevelArgs<TS, TW>& a) {
-  using C = LevelCfgM<TS, MODE>;
-  using G = LevelTile<C::NW, C::RPW>;
-  const int gx = (a.m[2] + G::BX - 1) / G::BX, gy = (a.m[1] + G::BY - 1) / G::BY;
-  const int chunks = choose_chunks(p, int64_t(gx) * gy, a.m[0], level_ctas_per_sm(C::NW), kLevelMaxChunk);
-  a.qz_chunk = (a.m[0] + chunks - 1) / chunks;
-  const int gz = (a.m[0] + a.qz_chunk - 1) / a.qz_chunk;
-  return dim3(gx, gy, gz);
+// Strip height and z chunk length of the level pass (sets a.rows, a.qz_chunk)
+// for `slices` grids of the level at once, `planes` coarse planes of each.  A warp streams rows + 2 units per
+// plane pair (the first and the last in part) over its chunk's planes and about
+// 1.2 more: long strips and chunks repeat least, short ones make more warps.
+// The model: with c warps on an SM a unit takes max(rate, chain / c) cycles of it,
+// `rate` what bounds the pass (FP64: 49 / 32 operations of 16 cycles; FP32: the
+// instructions and the shared-memory and shuffle pipe, measured at 513^3) and
+// `chain` one warp's own latency (measured with few warps).  Warps that are all
+// resident come in whole numbers per SM; more of them than fit run one after
+// another, with half a warp's time lost at the end.  FP32 strips have at most 10
+// rows: longer ones take the L1 cache's share of the memory (513^3: 0.29 ms with
+// 8 or 10 rows, 0.33 with 12 to 14).
+template <int MODE, typename TI, bool QZ, typename TS, typename TW>
+void level_shape(const mgr_plan* p, LevelArgs<TS, TW>& a, int64_t slices = 1, int planes = 1 << 30) {
+  const double rate = sizeof(TS) == 8 ? (MODE == 0 ? 784 : 512) : (MODE == 0 ? 110 : 62);
+  const double chain = sizeof(TS) == 8 ? (MODE == 0 ? 4200 : 2900) : (MODE == 0 ? 1000 : 620);
+  const int max_rows = sizeof(TS) == 8 ? 16 : 10;
+  const int mz = std::min(a.m[0], planes), my = a.m[1], mx = a.m[2];
+  const int64_t sms = p->ctx->num_sms;
+  double best = 1e300;
+  for (int rows = 1; rows <= max_rows; ++rows) {
+    const int strips = (my + rows - 1) / rows;
+    int r = (my + strips - 1) / strips;  // evenly over the strips
+    // FP32 codes: half a 14-row strip, whose places decide a rounding (see level_body)
+    const bool fixed = QZ && MODE == 0 && sizeof(TS) == 4;
+    if (fixed) r = 7;
+    const int64_t warps = level_warps<32>(mx, my, r) * slices;
+    const int64_t resident = std::min<int64_t>(
+        level_ctas<MODE, TS>(),
+        (int64_t(227) << 10) / (level_smem_bytes<MODE, TI, TS, QZ>(r, level_slot_rows(mx, my, r)) + 1024));
+    // every chunk length that splits the planes evenly, longest first
+    for (int len = mz;;) {
+      const int chunks = (mz + len - 1) / len;
+      const int even = (mz + chunks - 1) / chunks;
+      const int64_t w = warps * chunks;
+      const double units = (r + 1.5) * (even + (mz > 1 ? 1.2 : 0.0));
+      const bool all = w <= sms * resident;
+      const double loads = all ? double((w + sms - 1) / sms) : double(w) / sms + 0.5;
+      const double cost = units * loads * std::max(rate, chain / (all ? loads : double(resident)));
+      if (cost < best * (1 - 1e-9)) {
+        best = cost;
+        a.rows = r;
+        a.qz_chunk = even;
+      }
+      if (even <= 1) break;
+      len = even - 1;
+    }
+    if (rows >= my || fixed) break;
+  }
+}
+
+// Grid of the level pass: warps over the strips, z chunks (sets a.rows, a.qz_chunk;
+// chosen for `planes` coarse planes at a time).
+template <int MODE, typename TI, bool QZ, typename TS, typename TW>
+dim3 level_grid(const mgr_plan* p, LevelArgs<TS, TW>& a, int planes = 1 << 30) {
+  level_shape<MODE, TI, QZ>(p, a, 1, planes);
+  return dim3(unsigned(level_warps<32>(a.m[2], a.m[1], a.rows)), (a.m[0] + a.qz_chunk - 1) / a.qz_chunk);
+}
+
+// z chunks [c0, c1) of the level pass's grid (the grid level_grid chooses with
+// `planes`; c1 < 0: all of them): a level pass may run as several such launches,
+// each as soon as its input planes are ready.
+template <int MODE, typename TI, typename TD, typename TS, typename TW, bool PK, bool QZ = false>
+void launch_level_chunks(const mgr_plan* p, LevelArgs<TS, TW>& a, int c0, int c1, cudaStream_t st,
+                         int planes = 1 << 30) {
+  dim3 grid = level_grid<MODE, TI, QZ>(p, a, planes);
+  if (c1 < 0) c1 = int(grid.y);
+  if (c1 <= c0 || c1 > int(grid.y)) return;
+  const size_t sm = level_smem_bytes<MODE, TI, TS, QZ>(a.rows, level_slot_rows(a.m[2], a.m[1], a.rows));
+  auto kern = k_level<MODE, TI, TD, TS, TW, true, PK, QZ>;
+  if constexpr (!PK) {
+    if (a.s[2] != 1) kern = k_level<MODE, TI, TD, TS, TW, false, PK, QZ>;
+  }
+  raise_smem_limit(kern, sm);
+  // (the grid's y extent is limited to 65535)
+  for (int c = c0; c < c1; c += 65535) {
+    a.bz0 = c;
+    grid.y = unsigned(std::min(c1 - c, 65535));
+    kern<<<grid, 32, sm, st>>>(a);
+  }
+  a.bz0 = 0;
 }
 
 template <int MODE, typename TI, typename TD, typename TS, typename TW, bool PK, bool QZ = false>
 void launch_level(const mgr_plan* p, LevelArgs<TS, TW>& a, cudaStream_t st) {
-  using C = LevelCfgM<TS, MODE>;
-  constexpr size_t sm = level_smem_bytes<C::NW, C::RPW, C::STAGES, TI, TS>();
-  auto kern = k_level<MODE, C::NW, C::RPW, C::STAGES, TI, TD, TS, TW, PK, QZ>;
-  raise_smem_limit(kern, sm);
-  dim3 grid = level_grid<MODE>(p, a);
-  kern<<<grid, C::NW * 32, sm, st>>>(a);
-}
-
-// z chunks [c0, c1) of the level pass's grid (the grid level_grid chooses):
-// a level pass may run as several such launches, each as soon as its input
-// planes are ready.
-template <int MODE, typename TI, typename TD, typename TS, typename TW, bool PK, bool QZ = false>
-void launch_level_chunks(const mgr_plan* p, LevelArgs<TS, TW>& a, int c0, int c1, cudaStream_t st) {
-  using C = LevelCfgM<TS, MODE>;
-  constexpr size_t sm = level_smem_bytes<C::NW, C::RPW, C::STAGES, TI, TS>();
-  auto kern = k_level<MODE, C::NW, C::RPW, C::STAGES, TI, TD, TS, TW, PK, QZ>;
-  raise_smem_limit(kern, sm);
-  dim3 grid = level_grid<MODE>(p, a);
-  if (c1 <= c0 || c1 > int(grid.z)) return;
-  a.bz0 = c0;
-  grid.z = unsigned(c1 - c0);
-  kern<<<grid, C::NW * 32, sm, st>>>(a);
-  a.bz0 = 0;
+  launch_level_chunks<MODE, TI, TD, TS, TW, PK, QZ>(p, a, 0, -1, st);
 }
 
 // c: nodal coefficients (PK false), the packed class of level l (PK true), or

@@ -1,39 +1,48 @@
 // mgr_level.cuh -- the level pass of decomposition (coefficients + load
 // vector) and the load-vector pass of recomposition, for sm_103a.
 //
-// Per level l (level grid n -> coarse grid m), a CTA owns BX x BY coarse
-// (y, x) nodes and a chunk of coarse z planes.  It streams the fine z planes
-// of its region (the owned fine nodes plus the two-node halo the 5-tap
-// mass-transfer stencil needs) in pairs: the coarse-in-z plane p(t) and the
-// fine-in-z plane p(t)-1 between p(t-1) and p(t).
+// Per level l (level grid n -> coarse grid m), one warp owns a strip of coarse
+// y rows and a chunk of coarse z planes for the coarse x nodes of its lanes.
+// It streams the fine z planes of its region in pairs -- the coarse-in-z plane
+// p(t) and the fine-in-z plane between p(t-1) and p(t) -- and each plane pair in
+// units of row pairs: the coarse row p(qc) and the fine row above it.  No step
+// needs another warp, so there is no CTA barrier and no shared tile; a CTA is
+// one warp, and its plane and row bookkeeping is the same for all lanes.
 //
-// Thread mapping (fixed for the CTA's lifetime, so every per-row and
-// per-column weight and address is computed once): the CTA's threads form
-// row groups of LX lanes (a whole warp, LX = 32, or half of one, LX = 16:
-// a tile 14 coarse nodes wide, for fields whose coarse rows are short);
-// lane l of a group owns the fine column pair (rx0 + 2l, rx0 + 2l + 1) of
-// the region, group w owns RPW fine row pairs.  Below, "lane" and "warp"
-// are a thread's lane in its group and its group.  The region starts on a
-// coarse node, so the first node of every pair is coarse and the second is
-// the fine node between two coarse ones (or, at the end of an axis whose
-// length is even, the last coarse node).
+// Lanes.  Lane l owns one coarse x node and the fine node after it (two level
+// columns).  The nodes of all strips of the level, one strip after another,
+// form one sequence; a row group of LX lanes (a warp, or half of one) takes LX
+// consecutive entries and shares two of them with its neighbours, so that each
+// lane with outputs has its left and right neighbour in the group (warp
+// shuffles) whatever the level's width: 30 of 32 lanes produce outputs on every
+// grid, where tiles 30 nodes wide left almost half of them idle at 33.  Where a
+// strip ends inside a group, the neighbour from the other strip carries weight 0.
 //
-// Coefficients (Sec. II.A.1), separable and in the paper's FMA form
-// (Table "fma"): on a coarse-z plane the x interpolant of a coarse row uses
-// the right neighbour's value (warp shuffle), the y interpolant of a fine row
-// uses the next coarse row's interpolant (the next pair of the same thread,
-// or the next warp's first pair through shared memory); a fine-z plane
-// interpolates between the xy interpolants of its two coarse planes, which
-// each thread keeps in registers.
+// Coefficients (Sec. II.A.1), separable and in the paper's FMA form (Table
+// "fma"): the x interpolant of a coarse row uses the right neighbour's value; the
+// y interpolant of the fine row above lies between this coarse row's interpolants
+// and the previous one's (kept from the previous unit); a fine-z plane
+// interpolates between the xy interpolants of its two coarse planes, the first
+// plane's kept in the lane's own shared-memory slots, one per unit.
 //
-// Load vector f' = (x_k D_k^-1 K_k) c (Sec. II.A.2, III.A.2): c goes to
-// shared memory, the x stencil runs on rows (5 taps; in FP64 2 on rows that
-// are coarse in y and z, where c vanishes on coarse nodes), the y stencil on
-// the x results, and the z stencil accumulates in registers over the
-// streamed planes.  FP32 keeps the two planes interleaved in its tiles
-// ({coarse, fine} per node) and runs both planes' stencils as paired FMAs.
-// The per-plane-pair constants come from a table the CTA fills once.  Two
-// CTA barriers per plane pair.
+// Load vector f' = (x_k D_k^-1 K_k) c (Sec. II.A.2, III.A.2): the x stencil of
+// each row takes the neighbours' columns by shuffles (two taps on the rows coarse
+// in y and z, where c vanishes on coarse nodes); the y stencil of coarse row qc-1
+// is complete once unit qc's rows are there, from results kept in registers; the
+// z stencil accumulates over the planes in the lane's shared-memory slots.
+//
+// Loads.  Asynchronous 4- or 8-byte copies into a ring of units in shared memory,
+// three units ahead in FP32 (one in FP64): with the next unit's loads in
+// registers the FP32 pass waited for them (0.83 ms at 513^3, against 0.30).
+//
+// What bounds it.  FP64: the FP64 pipe, one SM-wide operation per 16 cycles and
+// warp; a unit takes 49 of them in decomposition, 32 in recomposition (level_shape
+// counts with that).  FP32: no single unit (at 513^3 issue slots 50%, shared-memory
+// and shuffle pipe 62%, DRAM 48%), but the dependent chains of about 12 warps per
+// SM.  513^3, finest level, against the earlier pass of 8-warp tiles with two CTA
+// barriers per plane pair: FP64 decomposition 2.12 -> 1.82 ms, recomposition 1.48
+// -> 1.12 ms; FP32 0.375 -> 0.303 and 0.248 -> 0.174 ms.  65^3 FP64, where the
+// tiles left most SMs without work: 49 -> 24 us.
 //
 // Coefficient addressing.  Nodal (PK = false): a coefficient sits at its node's
 // full-grid position.  Class-packed (PK = true, Sec. I coefficient classes): the
@@ -50,77 +59,6 @@
 // code * q_l; q_l is the bin width of the level's class.
 #pragma once
 
-template <int NW, int RPW, int LX = 32>
-struct LevelTile {
-  static_assert(LX == 32 || LX == 16, "row groups of a warp or half a warp");
-  static constexpr int NT = NW * 32;
-  static constexpr int NG = NT / LX;       // row groups
-  static constexpr int BX = LX - 2;        // coarse x outputs per CTA
-  static constexpr int BY = NG * RPW - 2;  // coarse y outputs per CTA
-  static constexpr int RC = 2 * LX;        // fine column slots (region width <= 2*BX+3 = RC-1)
-  static constexpr int RR = 2 * NG * RPW;  // fine row slots (region height <= 2*BY+3 = RR-1)
-  static constexpr int CP = RC + 2;        // c row pitch: even, so column pairs stay 8/16-byte aligned
-  // x-stencil result row pitch: with half-warp groups the two halves of a warp
-  // work 2*RPW rows apart, and a pitch of 4 (mod 8) words puts them in
-  // different banks
-  static constexpr int GP = LX == 32 ? 32 : LX + 4;
-};
-
-// Tile configuration of the level pass per stencil type: 8 warps with two
-// row pairs each (two CTAs per SM); FP64 uses a single cp.async stage (the
-// FP64 pipe, not memory latency, bounds it, and the smaller footprint keeps
-// two CTAs per SM), FP32 two stages.  The MGR_LEVEL_* macros override the
-// defaults at build time (tuning sweeps).
-#ifndef MGR_LEVEL_F64_NW
-#define MGR_LEVEL_F64_NW 8
-#endif
-#ifndef MGR_LEVEL_F64_RPW
-#define MGR_LEVEL_F64_RPW 2
-#endif
-#ifndef MGR_LEVEL_F64_STAGES
-#define MGR_LEVEL_F64_STAGES 1
-#endif
-#ifndef MGR_LEVEL_F32_NW
-#define MGR_LEVEL_F32_NW 8
-#endif
-#ifndef MGR_LEVEL_F32_RPW
-#define MGR_LEVEL_F32_RPW 2
-#endif
-#ifndef MGR_LEVEL_F32_STAGES
-#define MGR_LEVEL_F32_STAGES 2
-#endif
-template <typename TS>
-struct LevelCfg;
-template <>
-struct LevelCfg<double> {
-  static constexpr int NW = MGR_LEVEL_F64_NW, RPW = MGR_LEVEL_F64_RPW, STAGES = MGR_LEVEL_F64_STAGES;
-};
-template <>
-struct LevelCfg<float> {
-  static constexpr int NW = MGR_LEVEL_F32_NW, RPW = MGR_LEVEL_F32_RPW, STAGES = MGR_LEVEL_F32_STAGES;
-};
-
-// Tile configuration per pass: the recomposition load pass (MODE 1) computes
-// no coefficients and keeps fewer values per row pair in registers, so in FP32
-// it also fits three row pairs per warp (a taller tile, less repeated halo
-// work) within the same 128 registers; MGR_LEVEL_F32_REC_RPW selects it at
-// build time (measured: faster at 1000x700x300, slower at 513^3; default two).
-#ifndef MGR_LEVEL_F32_REC_RPW
-#define MGR_LEVEL_F32_REC_RPW 2
-#endif
-template <typename TS, int MODE>
-struct LevelCfgM {
-  static constexpr int NW = LevelCfg<TS>::NW, STAGES = LevelCfg<TS>::STAGES;
-  static constexpr int RPW = (MODE == 1 && sizeof(TS) == 4) ? MGR_LEVEL_F32_REC_RPW : LevelCfg<TS>::RPW;
-};
-
-// CTAs per SM a level-pass or interpolation CTA of NW warps is compiled for:
-// 16 warps per SM in every configuration, so each thread may use up to 128
-// registers.
-#ifndef MGR_LEVEL_CTAS_16W
-#define MGR_LEVEL_CTAS_16W 1
-#endif
-constexpr int level_ctas_per_sm(int nw) { return nw >= 16 ? MGR_LEVEL_CTAS_16W : 16 / nw; }
 template <typename T>
 struct Pair;
 template <>
@@ -198,22 +136,30 @@ __device__ __forceinline__ TS dequant(int k, TS q) {
   return code_value<TS>(k) * q;
 }
 
+// One axis of a level in "slots".  Coarse node q (level node p(q) = min(2q,
+// n-1)) owns two slots: its own, and the fine node p(q)+1 between q and q+1
+// when there is one.  The plan tabulates per coarse node the five weights of
+// its mass-transfer row on the slots (q-1).own, (q-1).fine, q.own, q.fine,
+// (q+1).own -- 0 where a slot does not exist -- and the interpolation weights
+// of q.fine (kSlot entries per node, filled by build_plan_tables).  In slots an
+// axis of even length, whose last two nodes are both coarse, and the ends of
+// an axis need no code of their own: their missing slots carry weight 0.
+constexpr int kSlotWa = 5, kSlotWb = 6;  // entries 0..4: the row's weights
+
 template <typename TS, typename TW>
 struct LevelArgs {
-  const void* in;  // DEC: level-l values; REC: nodal coefficients (full grid)
+  const void* in;  // DEC: level-l values (unit stride); REC: coefficients (nodal full grid, or the packed class)
   int64_t in_sz, in_sy;
-  int in_full;     // 1: `in` is addressed through the full-grid map min(i*s, N-1)
-  void* y;         // DEC: nodal output (full grid)
+  void* y;         // DEC: nodal output (full grid) or the packed class
   int64_t y_sz, y_sy;
   TW* w;           // DEC: coarse nodal values (compact m grid)
   TW* f;           // load vector (compact m grid)
   int64_t c_sz, c_sy;
   int n[3], m[3];
-  int64_t s[3], N[3];
-  const TS* wa[3];
-  const TS* wb[3];
-  const TS* k[3];
-  int qz_chunk;
+  int64_t s[3], N[3];   // full-grid map of a level-l node: min(i * s, N - 1)
+  const TS* slot[3];    // slot tables, kSlot entries per coarse node
+  int rows;        // coarse rows per strip
+  int qz_chunk;    // coarse planes per z chunk
   int bz0;         // first z chunk of this launch (a launch may cover a subset of the chunks)
   int write_y;
   double qs;                // QZ: 1/bin width (MODE 0) or bin width (MODE 1)
@@ -222,39 +168,545 @@ struct LevelArgs {
                             // 4D field that is fine in time), not only the fine ones
 };
 
-// FP64 keeps the x / y stencil weights in shared memory (the FP64 pass is
-// bound by the FP64 pipe and short of registers), FP32 in registers (its
-// pass is bound by instruction issue).
+// Units in flight per warp: a ring of units' rows in shared memory, filled by
+// asynchronous copies all but one ahead.  Two units in FP64, whose units take
+// over 3000 cycles of the FP64 pipe each, four in FP32.
 template <typename TS>
-constexpr bool weights_in_smem() {
-  return sizeof(TS) == 8;
+constexpr int level_ring() {
+  return sizeof(TS) == 8 ? 2 : 4;
+}
+// Row entries of a warp's y slot table: the rows of the strips its lanes can
+// belong to and two before them.
+__host__ __device__ inline int level_slot_rows(int mx, int my, int rows) {
+  const int strips = (my + rows - 1) / rows, span = 31 / mx + 2;
+  return (span < strips ? span : strips) * rows + 2;
+}
+// xy interpolants of a coarse plane that a lane keeps per unit.  FP64: four (both
+// columns of the coarse row and of the fine row above it).  FP32 keeps the
+// coarse row's two and forms the fine row's again from them (two FMAs and two
+// products; the smaller footprint lets 16 instead of 12 warps reside on an SM),
+// but for quantized output, whose fine rows have a rounding of their own.
+template <int MODE, typename TS, bool QZ>
+constexpr int level_interpolants() {
+  return MODE == 1 ? 0 : (sizeof(TS) == 4 && !QZ) ? 2 : 4;
+}
+// Shared memory of one warp: the ring (four rows of 32 column pairs a unit), per
+// unit (a strip of `rows` coarse rows has rows + 2) and lane the z accumulators
+// of two coarse planes and the interpolants of the last one, and the y slots of
+// its rows.
+template <int MODE, typename TI, typename TS, bool QZ = false>
+__host__ __device__ constexpr size_t level_smem_bytes(int rows, int slot_rows) {
+  return sizeof(TI) * level_ring<TS>() * 256 +
+         sizeof(TS) * (size_t(rows + 2) * 32 * (2 + level_interpolants<MODE, TS, QZ>()) + size_t(slot_rows) * kSlot);
 }
 
-// Plane pairs a level-pass CTA streams at most (its z chunk plus the halo
+// Lane groups of LX lanes over the coarse nodes of all strips of a level (strip
+// by strip, each mx long): group g holds positions g*(LX-2) .. g*(LX-2)+LX-1,
+// its first and last lanes only as neighbours.
+template <int LX>
+__host__ __device__ inline int64_t level_groups(int mx, int my, int rows) {
+  const int64_t total = int64_t((my + rows - 1) / rows) * mx;
+  return total <= LX ? 1 : (total - 2 + LX - 3) / (LX - 2);
+}
+template <int LX>
+__host__ __device__ inline int64_t level_warps(int mx, int my, int rows) {
+  return (level_groups<LX>(mx, my, rows) + 32 / LX - 1) / (32 / LX);
+}
+
+template <typename TS>
+struct Slots {
+  TS k0, k1, k2, k3, k4, wa, wb;
+};
+template <typename TS>
+__device__ __forceinline__ Slots<TS> load_slots(const TS* t, int q);
+template <>
+__device__ __forceinline__ Slots<float> load_slots<float>(const float* t, int q) {
+  const float4* p = reinterpret_cast<const float4*>(t) + 2 * q;
+  const float4 a = p[0], b = p[1];
+  return Slots<float>{a.x, a.y, a.z, a.w, b.x, b.y, b.z};
+}
+template <>
+__device__ __forceinline__ Slots<double> load_slots<double>(const double* t, int q) {
+  const double2* p = reinterpret_cast<const double2*>(t) + 4 * q;
+  const double2 a = p[0], b = p[1], c = p[2], d = p[3];
+  return Slots<double>{a.x, a.y, b.x, b.y, c.x, c.y, d.x};
+}
+
+// Values of the coarse and the fine plane of a pair: FP32 runs both planes'
+// stencils as paired FMAs (per plane the same operations as scalar ones).
+template <typename TS>
+struct Planes {
+  TS c, f;
+};
+// Five-tap sum in slot order, of both planes (HF) or of the coarse plane alone.
+template <bool HF>
+__device__ __forceinline__ Planes<double> taps(const Slots<double>& w, Planes<double> a, Planes<double> b,
+                                               Planes<double> c, Planes<double> d, Planes<double> e) {
+  Planes<double> r;
+  r.c = fma(w.k4, e.c, fma(w.k3, d.c, fma(w.k2, c.c, fma(w.k1, b.c, w.k0 * a.c))));
+  r.f = HF ? fma(w.k4, e.f, fma(w.k3, d.f, fma(w.k2, c.f, fma(w.k1, b.f, w.k0 * a.f)))) : 0.0;
+  return r;
+}
+template <bool HF>
+__device__ __forceinline__ Planes<float> taps(const Slots<float>& w, Planes<float> a, Planes<float> b,
+                                              Planes<float> c, Planes<float> d, Planes<float> e) {
+  if constexpr (HF) {
+    float2 g = __fmul2_rn(make_float2(w.k0, w.k0), make_float2(a.c, a.f));
+    g = __ffma2_rn(make_float2(w.k1, w.k1), make_float2(b.c, b.f), g);
+    g = __ffma2_rn(make_float2(w.k2, w.k2), make_float2(c.c, c.f), g);
+    g = __ffma2_rn(make_float2(w.k3, w.k3), make_float2(d.c, d.f), g);
+    g = __ffma2_rn(make_float2(w.k4, w.k4), make_float2(e.c, e.f), g);
+    return Planes<float>{g.x, g.y};
+  } else {
+    return Planes<float>{fmaf(w.k4, e.c, fmaf(w.k3, d.c, fmaf(w.k2, c.c, fmaf(w.k1, b.c, w.k0 * a.c)))), 0.f};
+  }
+}
+template <int LX, bool HF, typename TS>
+__device__ __forceinline__ Planes<TS> from_left(Planes<TS> v) {
+  return Planes<TS>{__shfl_up_sync(0xffffffffu, v.c, 1, LX), HF ? __shfl_up_sync(0xffffffffu, v.f, 1, LX) : TS(0)};
+}
+template <int LX, bool HF, typename TS>
+__device__ __forceinline__ Planes<TS> from_right(Planes<TS> v) {
+  return Planes<TS>{__shfl_down_sync(0xffffffffu, v.c, 1, LX), HF ? __shfl_down_sync(0xffffffffu, v.f, 1, LX) : TS(0)};
+}
+
+// One warp's work: lane groups bx*32/LX .. and z chunk bz of level args `a`.
+// PK: coefficients in the class-packed layout (MODE 0 writes `y`, MODE 1 reads
+// `in` as the class of this level; y_sz / in_sz = n1*n2, y_sy / in_sy = n2).
+// QZ (with PK): those coefficients are int32 codes (TD = int in MODE 0, TI =
+// int in MODE 1).
+// S1: the coefficients lie at unit stride (the finest level of the nodal layout;
+// always when packed).
+// AF: honour `all_fine` (the 4D form's time slices; a runtime flag read once).
+template <int MODE, typename TI, typename TD, typename TS, typename TW, bool S1, bool PK = false, bool QZ = false,
+          bool AF = false, int LX = 32>
+__device__ __forceinline__ void level_body(const LevelArgs<TS, TW>& a, int bx, int bz, unsigned char* smem_raw) {
+  static_assert(LX == 32 || LX == 16, "lane groups of a warp or half a warp");
+  static_assert(S1 || !PK, "a packed class has unit stride");
+  using TS2 = typename Pair<TS>::type;
+  using TI2 = typename Pair<TI>::type;
+  using P = Planes<TS>;
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr int IPN = level_interpolants<MODE, TS, QZ>(), RING = level_ring<TS>();
+  // unit-stride input columns: the level's values (MODE 0), or unit-stride coefficients
+  constexpr bool U1 = MODE == 0 || S1;
+  // FP32 also computes what the first two units of a plane leave unused, instead
+  // of branching around it; FP64, bound by its pipe, skips it
+  constexpr bool SKIP = sizeof(TS) == 8;
+  const int lid = threadIdx.x & 31, lane = lid % LX;
+  const int nz = a.n[0], ny = a.n[1], nx = a.n[2];
+  const int mz = a.m[0], my = a.m[1], mx = a.m[2];
+  const int rows = a.rows;
+  const int total = ((my + rows - 1) / rows) * mx;
+  const int group = bx * (32 / LX) + lid / LX;
+  const int pos = group * (LX - 2) + lane;
+  const bool out = pos < total && (lane > 0 || group == 0) && (lane < LX - 1 || pos == total - 1);
+  const int strip = min(pos, total - 1) / mx;
+  const int q = min(pos, total - 1) - strip * mx;
+  const int qy0 = strip * rows;
+  const int nrow = min(rows, my - qy0);
+  const int units = __reduce_max_sync(FULL, nrow) + 2;
+  const int qz0 = bz * a.qz_chunk, qz1 = min(qz0 + a.qz_chunk, mz);
+  const int t_start = max(qz0 - 1, 0), t_end = min(qz1, mz - 1);
+
+  const TI* __restrict__ in = static_cast<const TI*>(a.in);
+  TD* __restrict__ yout = static_cast<TD*>(a.y);
+  // bounds-checking builds: extents (elements) of the buffers this warp
+  // addresses; the LVL_* forms below check against them (other builds run the
+  // plain accesses)
+#ifdef MGR_DEBUG_BOUNDS
+  const long long n_in = MODE == 0 ? (long long)nz * a.in_sz
+                         : PK      ? (long long)nz * a.in_sz - (long long)mz * a.c_sz
+                                   : (long long)a.N[0] * a.in_sz;
+  const long long n_y = PK ? (long long)nz * a.y_sz - (long long)mz * a.c_sz : (long long)a.N[0] * a.y_sz;
+  const long long n_c = (long long)mz * a.c_sz;
+#endif
+#define LVL_CP(dst, src) \
+  MGR_GUARD(MGR_PIN(src, in, n_in, kDbgLevelIn) && MGR_PIN(dst, ring, RING * 256, kDbgLevelStage), \
+            cp_async(dst, src, int(sizeof(TI))))
+#define LVL_Y(p, v) MGR_GUARD(MGR_PIN(p, yout, n_y, kDbgLevelY), *(p) = (v))
+#define LVL_W(p, v) MGR_GUARD(MGR_PIN(p, a.w, n_c, kDbgLevelW), *(p) = (v))
+#define LVL_F(p, v) MGR_GUARD(MGR_PIN(p, a.f, n_c, kDbgLevelF), *(p) = (v))
+  const bool afine = AF && MODE == 1 && a.all_fine;
+  const TS qs = QZ ? TS(a.qs) : TS(1);
+  // value written for coefficient v (MODE 0); value of a read coefficient
+  // (MODE 1; with QZ the code itself: the bin width scales the load vector
+  // once per coarse node instead, see fout)
+  auto yval = [&](TS v) -> TD {
+    if constexpr (QZ) return TD(quant_code(v, qs, a.qsat));
+    else return TD(v);
+  };
+  auto cval = [&](TI v) -> TS {
+    if constexpr (QZ && MODE == 1) return code_value<TS>(int(v));
+    else return TS(v);
+  };
+  auto fout = [&](TS acc) -> TW {
+    if constexpr (QZ && MODE == 1) return TW(acc) * TW(a.qs);
+    else return TW(acc);
+  };
+
+  // ---- this lane's column: own node and, when fx, the fine node after it
+  const Slots<TS> kx = load_slots<TS>(a.slot[2], q);
+  const bool fx = 2 * q + 1 < nx - 1;
+  // input columns.  Unit stride: the pair (c, c+1), c = 2q; the axis' last node
+  // has no right neighbour and reads (n-2, n-1), its own value second (swp).
+  // Strided: own node, and the fine node or, where there is none, the own node
+  // again.  A slot without a node holds some value of the row and meets weight 0.
+  const bool swp = U1 && 2 * q >= nx - 1;
+  const int ic0 = U1 ? min(2 * q, nx - 2) : int(min(2 * int64_t(q) * a.s[2], a.N[2] - 1));
+  const int64_t icd = U1 ? 1 : (fx ? a.s[2] : 0);
+  // output columns (MODE 0)
+  const int yc0 = PK ? min(2 * q, nx - 1) : int(min(2 * int64_t(q) * a.s[2], a.N[2] - 1));
+  const int64_t ycd = S1 ? 1 : a.s[2];
+  // rows: row i of the level sits at min(i * stride, length - 1) * pitch, in
+  // (r) the input and (o) the output
+  const int rs = U1 ? 1 : int(a.s[1]), rN = U1 ? ny : int(a.N[1]), isy = int(a.in_sy);
+  const int os = S1 ? 1 : int(a.s[1]), oN = S1 ? ny : int(a.N[1]), ysy = int(a.y_sy);
+  const int csy = int(a.c_sy);
+
+  // z plane offsets (in: level plane g; coarse planes are g = p(t))
+  auto iplane = [&](int g) -> int64_t {
+    if (PK && MODE == 1) return int64_t(g) * a.in_sz - int64_t(cidx(g)) * a.c_sz;
+    return U1 ? int64_t(g) * a.in_sz : fmap(g, a.s[0], a.N[0]) * a.in_sz;
+  };
+  auto yplane = [&](int g) -> int64_t {
+    if (PK) return int64_t(g) * a.y_sz - int64_t(cidx(g)) * a.c_sz;
+    return S1 ? int64_t(g) * a.y_sz : fmap(g, a.s[0], a.N[0]) * a.y_sz;
+  };
+  auto has_fine = [&](int t) { return t > t_start && pidx(t, nz) - pidx(t - 1, nz) == 2; };
+
+  // ---- shared memory: ring, z accumulators, interpolants, y slots
+  TI* ring = reinterpret_cast<TI*>(smem_raw);                               // [ring][4 rows][own, fine column][32 lanes]
+  TS* acc_s = reinterpret_cast<TS*>(ring + RING * 256);               // [units][32][2]
+  TS* ip_s = acc_s + (rows + 2) * 64;                                       // [units][32][IPN]
+  TS* ky_s = ip_s + (rows + 2) * 32 * IPN;                                  // [slot rows][kSlot]
+  {
+    // rows qy0 - 2 of the first lane's strip on; rows outside the grid have weights 0
+    const int first_row = __shfl_sync(FULL, qy0, 0) - 2, n = level_slot_rows(mx, my, rows);
+    for (int i = lid; i < n * kSlot; i += 32) {
+      const int row = first_row + i / kSlot;
+      ky_s[i] = (row >= 0 && row < my) ? a.slot[1][int64_t(row) * kSlot + i % kSlot] : TS(0);
+    }
+    __syncwarp();
+    ky_s += (qy0 - 2 - first_row) * kSlot;  // this lane's unit 0
+  }
+
+  // ---- copies of the next unit (unit lu of plane pair lt) into the ring slot at
+  // d0 / d1 (own / fine column).  Rows cr, cs, fr, fs: the coarse row p(qc) and
+  // the fine row above it, in the coarse plane and the fine plane; rows outside
+  // the grid read some row of it and carry weight 0
+  int lt = t_start, lu = 0, lslot = 0;
+  const int lrow0 = 2 * (qy0 - 1) * rs * isy, lrow_max = (rN - 1) * isy;
+  int lrow = lrow0;
+  bool lhf = false;
+  const TI *lc = nullptr, *lf = nullptr;
+  auto load_planes = [&]() {
+    const int p = pidx(lt, nz);
+    lhf = has_fine(lt);
+    lc = in + iplane(p) + ic0;
+    lf = lhf ? in + iplane(p - 1) + ic0 : lc;
+  };
+  TI* const ring0 = ring + lid + (swp ? 32 : 0);
+  TI* const ring1 = ring + lid + (swp ? 0 : 32);
+  auto load_unit = [&]() {
+    if (lt <= t_end) {
+      TI* d0 = ring0 + lslot * 256;
+      TI* d1 = ring1 + lslot * 256;
+      TI* dx = ring + lslot * 256 + lid + 32;  // the fine column's slot
+      // element offsets of the two rows, clamped into the plane
+      const int r = min(max(lrow, 0), lrow_max), s = min(max(lrow - rs * isy, 0), lrow_max);
+      lrow += 2 * rs * isy;
+      if constexpr (PK && MODE == 1) {
+        // rows of a coarse plane: the coarse row holds its fine columns only
+        // (slots without a value: 0, they meet weights 0)
+        const int qc = min(max(qy0 - 1 + lu, 0), my - 1);
+        if (fx) LVL_CP(dx, lc - ic0 + (r - qc * mx + q));
+        else *dx = TI(0);
+        if (2 * qc - 1 < ny - 1 && qc > 0) {
+          const int o = (2 * qc - 1) * nx - qc * mx;
+          LVL_CP(d0 + 64, lc + o);
+          LVL_CP(d1 + 64, lc + o + 1);
+        } else {
+          d0[64] = d1[64] = TI(0);
+        }
+        if (lhf) {
+          LVL_CP(d0 + 128, lf + r);
+          LVL_CP(d1 + 128, lf + r + 1);
+          LVL_CP(d0 + 192, lf + s);
+          LVL_CP(d1 + 192, lf + s + 1);
+        }
+      } else {
+        const TI *pr = lc + r, *ps = lc + s;
+        if (MODE == 0 || AF) {
+          LVL_CP(d0, pr);
+          LVL_CP(d1, pr + icd);
+        } else {
+          LVL_CP(dx, swp ? pr : pr + icd);  // (the own column holds no coefficient)
+        }
+        if (!SKIP || lu > 0) {
+          LVL_CP(d0 + 64, ps);
+          LVL_CP(d1 + 64, ps + icd);
+        }
+        if (lhf) {
+          const TI *fr = lf + r, *fs = lf + s;
+          LVL_CP(d0 + 128, fr);
+          LVL_CP(d1 + 128, fr + icd);
+          if (!SKIP || lu > 0) {
+            LVL_CP(d0 + 192, fs);
+            LVL_CP(d1 + 192, fs + icd);
+          }
+        }
+      }
+      lslot = (lslot + 1) & (RING - 1);
+      if (++lu == units) {
+        lu = 0;
+        lrow = lrow0;
+        ++lt;
+        if (lt <= t_end) load_planes();
+      }
+    }
+    cp_commit();
+  };
+  load_planes();
+#pragma unroll
+  for (int i = 0; i < RING - 1; ++i) load_unit();
+  int slot = 0;  // ring slot of the unit being processed
+  // (QZ, FP32) parity of qc below the fine rows with the other rounding: row pairs
+  // count from the one before the 14-row strip that this strip is part of, from
+  // its first one in the first of them, and from two before where it starts on
+  // the last node of an axis of even length
+  const int qy14 = qy0 - qy0 % 14;
+  const int qz_parity = (qy14 + ((qy14 == 0 || (qy14 == my - 1 && (ny & 1) == 0)) ? 0 : 1)) & 1;
+  // rows with outputs, by unit: coarse rows u - 1 < nr, fine rows u - 2 < ns, all
+  // 0 on lanes without outputs
+  const unsigned nr = out ? nrow : 0, ns = out ? min(nrow, max((ny - 1) / 2 - qy0, 0)) : 0;
+  const unsigned nrx = fx ? nr : 0, nsx = fx ? ns : 0;  // at the fine column
+
+  // ---- one plane pair (HF: with a fine plane)
+  auto plane_pair = [&](auto hf_c, int t) {
+    constexpr bool HF = decltype(hf_c)::value;
+    const int Pc = pidx(t, nz);
+    const bool own_c = t >= qz0 && t < qz1, own_f = HF && t > qz0;
+    const bool wy_c = own_c && a.write_y, wy_f = own_f && a.write_y;  // coefficients written
+    TD* yzc = MODE == 0 ? yout + yplane(Pc) + yc0 : nullptr;
+    TD* yzf = MODE == 0 ? yout + yplane(HF ? Pc - 1 : Pc) + yc0 : nullptr;
+    // coarse values of this plane and load vector of the plane before it, at the unit's row
+    TW* wp = MODE == 0 ? a.w + (int64_t(t) * a.c_sz + (int64_t(qy0) - 1) * csy + q) : nullptr;
+    TW* fp = a.f + (int64_t(t - 1) * a.c_sz + (int64_t(qy0) - 2) * csy + q);
+    const unsigned nf = (t - 1 >= qz0 && t - 1 < qz1) ? nr : 0;       // plane t-1 complete
+    const unsigned nl = (t == mz - 1 && t < qz1) ? nr : 0;            // the last plane, too
+    // z weights of the two planes for the coarse planes t-1, t, t+1, and of the fine plane's interpolant
+    const TS* zt = a.slot[0] + int64_t(kSlot) * t;
+    const TS wzc0 = t > 0 ? zt[4 - kSlot] : TS(0), wzf0 = HF ? zt[3 - kSlot] : TS(0);
+    const TS wzc1 = zt[2], wzf1 = HF ? zt[1] : TS(0);
+    const TS wzc2 = t + 1 < mz ? zt[kSlot] : TS(0);
+    const TS za = (MODE == 0 && HF) ? zt[kSlotWa - kSlot] : TS(0), zb = (MODE == 0 && HF) ? zt[kSlotWb - kSlot] : TS(0);
+    const bool first = t == t_start;
+
+    // x-stencil results of the rows before: (qc-2).own, (qc-2).fine, (qc-1).own
+    P ga{}, gb{}, gc{};
+    TS i0p = TS(0), i1p = TS(0);  // x interpolants of coarse row qc-1 in this plane
+    TS j0p = TS(0), j1p = TS(0);  // and in the coarse plane before (IPN == 2)
+    int qc = qy0 - 1;
+    TS* ip = ip_s + lid * IPN;
+    TS2* ap = reinterpret_cast<TS2*>(acc_s + lid * 2);
+    const TS* kp = ky_s;
+    // output rows (element offsets): the coarse row and the fine row above it
+    int orow = 2 * qc * os * ysy;
+    const int orow_max = (oN - 1) * ysy;
+#pragma unroll 2
+    for (int u = 0; u < units; ++u, ++qc) {
+      // each lane copies, and reads, only its own slots of the ring
+      load_unit();
+      cp_wait<RING - 1>();
+      const TI* d = ring + slot * 256 + lid;
+      slot = (slot + 1) & (RING - 1);
+      const TI2 vcr{d[0], d[32]}, vcs{d[64], d[96]};
+      TI2 vfr{}, vfs{};
+      if constexpr (HF) {
+        vfr = TI2{d[128], d[160]};
+        vfs = TI2{d[192], d[224]};
+      }
+      // weights of coarse row qc-1: its stencil row and its fine row's interpolation
+      const Slots<TS> ky = load_slots<TS>(kp, 0);
+      kp += kSlot;
+
+      // ---- coefficients, own (0) and fine (1) column: coarse row (r), fine row above it (s)
+      P r0{}, r1{}, s0{}, s1{};
+      if constexpr (MODE == 0) {
+        const TS v0 = cval(vcr.x);
+        const TS vr = __shfl_down_sync(FULL, v0, 1, LX);
+        const TS i0 = v0;
+        TS i1 = fx ? fma(kx.wb, vr, kx.wa * v0) : TS(0);
+        TS i1n = i1;  // as the lower neighbour of the fine row
+        if constexpr (QZ && sizeof(TS) == 4) {
+          // FP32 codes are whole numbers that show the last bit of a coefficient, and
+          // they keep the values they have always had: there the interpolant was
+          // rounded the other way round on the last row of an axis of even length
+          // and below every second fine row of a strip of 14
+          const TS other = fx ? fma(kx.wa, v0, kx.wb * vr) : TS(0);
+          if (qc == my - 1 && (ny & 1) == 0) i1 = other;
+          if ((qc & 1) == qz_parity) i1n = other;
+        }
+        const TS i2 = fma(ky.wa, i0p, ky.wb * i0), i3 = fma(ky.wa, i1p, ky.wb * i1n);
+        r1.c = cval(vcr.y) - i1;
+        s0.c = cval(vcs.x) - i2;
+        s1.c = cval(vcs.y) - i3;
+        if constexpr (IPN == 2) {
+          if constexpr (HF) {
+            const float2 p = *reinterpret_cast<const float2*>(ip);
+            const TS p2 = fma(ky.wa, j0p, ky.wb * p.x), p3 = fma(ky.wa, j1p, ky.wb * p.y);
+            r0.f = cval(vfr.x) - za * p.x - zb * i0;
+            r1.f = cval(vfr.y) - za * p.y - zb * i1;
+            s0.f = cval(vfs.x) - za * p2 - zb * i2;
+            s1.f = cval(vfs.y) - za * p3 - zb * i3;
+            j0p = p.x;
+            j1p = p.y;
+          }
+          *reinterpret_cast<float2*>(ip) = make_float2(i0, i1);
+        } else {
+          if constexpr (HF) {
+            const TS2 p = *reinterpret_cast<const TS2*>(ip), pp = *reinterpret_cast<const TS2*>(ip + 2);
+            r0.f = cval(vfr.x) - za * p.x - zb * i0;
+            r1.f = cval(vfr.y) - za * p.y - zb * i1;
+            s0.f = cval(vfs.x) - za * pp.x - zb * i2;
+            s1.f = cval(vfs.y) - za * pp.y - zb * i3;
+          }
+          *reinterpret_cast<TS2*>(ip) = TS2{i0, i1};
+          *reinterpret_cast<TS2*>(ip + 2) = TS2{i2, i3};
+        }
+        ip += 32 * IPN;
+        i0p = i0;
+        i1p = i1;
+      } else {
+        r0.c = afine ? cval(vcr.x) : TS(0);
+        r1.c = cval(vcr.y);
+        s0.c = cval(vcs.x);
+        s1.c = cval(vcs.y);
+        if constexpr (HF) {
+          r0.f = cval(vfr.x);
+          r1.f = cval(vfr.y);
+          s0.f = cval(vfs.x);
+          s1.f = cval(vfs.y);
+        }
+      }
+
+      // ---- coefficient and coarse-value outputs
+      if constexpr (MODE == 0) {
+        const unsigned ur = unsigned(u - 1), us = unsigned(u - 2);
+        const bool wr = ur < nr, wrx = ur < nrx, ws = us < ns, wsx = us < nsx;
+        const int oc = min(orow, orow_max), osr = orow - os * ysy;
+        if (own_c && wr) LVL_W(wp, TW(vcr.x));
+        wp += csy;
+        orow += 2 * os * ysy;
+        if (wy_c) {
+          if constexpr (PK) {
+            // rows of a coarse plane leave the coarse nodes out: the coarse row keeps its fine columns
+            const int out_c = qc * mx;
+            if (wrx) LVL_Y(yzc + (oc - out_c + q - yc0), yval(r1.c));
+            if (ws) LVL_Y(yzc + (osr - out_c), yval(s0.c));
+            if (wsx) LVL_Y(yzc + (osr - out_c) + 1, yval(s1.c));
+          } else {
+            // (all-coarse nodes get a placeholder that a coarser level overwrites:
+            // at unit stride it keeps the row's sectors fully written)
+            TD *pr = yzc + oc, *ps = yzc + osr;
+            if (S1 && wr) LVL_Y(pr, TD(0));
+            if (wrx) LVL_Y(pr + ycd, TD(r1.c));
+            if (ws) LVL_Y(ps, TD(s0.c));
+            if (wsx) LVL_Y(ps + ycd, TD(s1.c));
+          }
+        }
+        if (HF && wy_f) {
+          TD *pr = yzf + oc, *ps = yzf + osr;
+          if (wr) LVL_Y(pr, yval(r0.f));
+          if (wrx) LVL_Y(pr + ycd, yval(r1.f));
+          if (ws) LVL_Y(ps, yval(s0.f));
+          if (wsx) LVL_Y(ps + ycd, yval(s1.f));
+        }
+      }
+
+      // ---- x stencil of the unit's rows (the coefficients of the coarse plane's
+      // coarse row vanish on coarse nodes)
+      P gd{}, ge;
+      if (!SKIP || u > 0) gd = taps<HF>(kx, from_left<LX, HF>(s0), from_left<LX, HF>(s1), s0, s1, from_right<LX, HF>(s0));
+      if constexpr (sizeof(TS) == 8) {
+        const P l1 = from_left<LX, HF>(r1);
+        if (AF && afine) {
+          ge = taps<HF>(kx, from_left<LX, HF>(r0), l1, r0, r1, from_right<LX, HF>(r0));
+        } else {
+          ge.c = fma(kx.k3, r1.c, kx.k1 * l1.c);
+          ge.f = HF ? fma(kx.k4, __shfl_down_sync(FULL, r0.f, 1, LX),
+                          fma(kx.k3, r1.f, fma(kx.k2, r0.f, fma(kx.k1, l1.f, kx.k0 * __shfl_up_sync(FULL, r0.f, 1, LX)))))
+                    : TS(0);
+        }
+      } else {
+        P l0{}, e0{};
+        if (AF && afine) {
+          l0 = from_left<LX, HF>(r0);
+          e0 = from_right<LX, HF>(r0);
+        } else if constexpr (HF) {
+          l0.f = __shfl_up_sync(FULL, r0.f, 1, LX);
+          e0.f = __shfl_down_sync(FULL, r0.f, 1, LX);
+        }
+        ge = taps<HF>(kx, l0, from_left<LX, HF>(r1), r0, r1, e0);
+      }
+
+      // ---- y stencil of coarse row qc-1 and its z accumulation
+      if (!SKIP || u > 1) {
+        TS2 acc = *ap;
+        if (first) acc.x = acc.y = TS(0);
+        const P g = taps<HF>(ky, ga, gb, gc, gd, ge);
+        acc.x = fma(wzc0, g.c, acc.x);
+        acc.y = fma(wzc1, g.c, acc.y);
+        const TS a2 = wzc2 * g.c;
+        if constexpr (HF) {
+          acc.x = fma(wzf0, g.f, acc.x);
+          acc.y = fma(wzf1, g.f, acc.y);
+        }
+        *ap = TS2{acc.y, a2};
+        if (unsigned(u - 2) < nf) LVL_F(fp, fout(acc.x));
+        if (unsigned(u - 2) < nl) LVL_F(fp + a.c_sz, fout(acc.y));
+      }
+      ap += 32;
+      fp += csy;
+      ga = gc;
+      gb = gd;
+      gc = ge;
+    }
+  };
+  for (int t = t_start; t <= t_end; ++t) {
+    if (has_fine(t)) plane_pair(std::true_type{}, t);
+    else plane_pair(std::false_type{}, t);
+  }
+}
+
+#undef LVL_CP
+#undef LVL_Y
+#undef LVL_W
+#undef LVL_F
+
+// Warps per SM the pass is compiled for: 16 (128 registers a thread), but 12 (168) for
+// the FP64 decomposition.
+template <int MODE, typename TS>
+constexpr int level_ctas() {
+  return MODE == 0 && sizeof(TS) == 8 ? 12 : 16;
+}
+
+template <int MODE, typename TI, typename TD, typename TS, typename TW, bool S1, bool PK, bool QZ>
+__global__ void __launch_bounds__(32, level_ctas<MODE, TS>()) k_level(const LevelArgs<TS, TW> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  level_body<MODE, TI, TD, TS, TW, S1, PK, QZ>(a, blockIdx.x, blockIdx.y + a.bz0, smem_raw);
+}
+
+// CTAs per SM an interpolation CTA of NW warps is compiled for: 16 warps per SM
+// in every configuration, so each thread may use up to 128 registers.
+constexpr int level_ctas_per_sm(int nw) { return nw >= 16 ? 1 : 16 / nw; }
+
+// Plane pairs an interpolation CTA streams at most (its z chunk plus the halo
 // planes before it): the per-plane-pair constants are tabulated once per CTA
 // in shared memory, so the hosts cap the chunk length at kLevelMaxChunk.
 constexpr int kLevelPlanes = 64;
 constexpr int kLevelMaxChunk = kLevelPlanes - 2;
-
-// Byte offset of the plane table in the level pass's shared memory (after the
-// stage buffers, coefficient tiles, x-stencil results and weights).
-template <int NW, int RPW, int STAGES, typename TI, typename TS, int LX = 32>
-constexpr size_t level_table_offset() {
-  using G = LevelTile<NW, RPW, LX>;
-  return (sizeof(TI) * STAGES * 2 * G::RR * G::RC +
-          sizeof(TS) * (2 * G::RR * G::CP + 2 * G::RR * G::GP + 5 * LX + 5 * G::NG * RPW +
-                        (sizeof(TS) == 8 ? G::NG * G::RC : 0)) +
-          15) / 16 * 16;
-}
-// per plane pair: four plane offsets (int64), eight weights (TS), a flag (int)
-template <typename TS>
-constexpr size_t level_table_bytes() {
-  return kLevelPlanes * (4 * sizeof(int64_t) + 8 * sizeof(TS) + sizeof(int));
-}
-template <int NW, int RPW, int STAGES, typename TI, typename TS, int LX = 32>
-constexpr size_t level_smem_bytes() {
-  return level_table_offset<NW, RPW, STAGES, TI, TS, LX>() + level_table_bytes<TS>();
-}
 
 // Copy the element pair (c0, c0+1) of one row into shared memory: one
 // 2-element cp.async when both are in the region, adjacent in memory and
@@ -290,744 +742,6 @@ __device__ __forceinline__ void store_pair(T* p0, T* p1, T a0, T a1, bool w0, bo
     if (w0) *p0 = a0;
     if (w1) *p1 = a1;
   }
-}
-
-// One CTA's work: coarse tile (bx, by) and z chunk bz of level args `a`,
-// with `smem_raw` the CTA's dynamic shared memory (level_smem_bytes).
-// PK: coefficients in the class-packed layout (MODE 0 writes `y`, MODE 1 reads
-// `in` as the class of this level; y_sz / in_sz = n1*n2, y_sy / in_sy = n2).
-// QZ (with PK): those coefficients are int32 codes (TD = int in MODE 0, TI =
-// int in MODE 1).
-// AF: honour `all_fine` (the 4D form's time slices; a runtime flag read once).
-// LX: lanes per row group (32 or 16).
-template <int MODE, int NW, int RPW, int STAGES, typename TI, typename TD, typename TS, typename TW, bool PK = false,
-          bool QZ = false, bool AF = false, int LX = 32>
-__device__ __forceinline__ void level_body(const LevelArgs<TS, TW>& a, int bx, int by, int bz,
-                                           unsigned char* smem_raw) {
-  using G = LevelTile<NW, RPW, LX>;
-  using TS2 = typename Pair<TS>::type;
-  using TI2 = typename Pair<TI>::type;
-  constexpr int RR = G::RR, RC = G::RC, CP = G::CP, GP = G::GP, NG = G::NG;
-  constexpr unsigned FULL = 0xffffffffu;
-  TI* stage = reinterpret_cast<TI*>(smem_raw);                                       // [STAGES][2][RR][RC]
-  TS* cbuf = reinterpret_cast<TS*>(smem_raw + sizeof(TI) * STAGES * 2 * RR * RC);  // [2][RR][CP]
-  TS* gxb = cbuf + 2 * RR * CP;                                                     // [2][RR][GP]
-  TS* kxs = gxb + 2 * RR * GP;                                                      // [5][LX]
-  TS* kys = kxs + 5 * LX;                                                           // [5][NG*RPW]
-  TS* xch = kys + 5 * NG * RPW;  // [NG][RC] FP64 only: x interpolants of each group's first coarse row
-  // plane table (kLevelPlanes entries): offsets of the input's coarse and fine
-  // planes and of the output's; weights wzc[3], wzf[2], za, zb; has-fine flag
-  int64_t* ptab = reinterpret_cast<int64_t*>(smem_raw + level_table_offset<NW, RPW, STAGES, TI, TS, LX>());
-  TS* pwt = reinterpret_cast<TS*>(ptab + 4 * kLevelPlanes);
-  int* pfl = reinterpret_cast<int*>(pwt + 8 * kLevelPlanes);
-
-  const int lane = threadIdx.x % LX, warp = threadIdx.x / LX;  // lane in the row group, row group
-  const int nz = a.n[0], ny = a.n[1], nx = a.n[2];
-  const int mz = a.m[0], my = a.m[1], mx = a.m[2];
-  const int qx0 = bx * G::BX, qx1 = min(qx0 + G::BX, mx);
-  const int qy0 = by * G::BY, qy1 = min(qy0 + G::BY, my);
-  const int qz0 = bz * a.qz_chunk, qz1 = min(qz0 + a.qz_chunk, mz);
-  const int rx0 = max(region_start(qx0, nx), 0), rx1 = min(pidx(qx1 - 1, nx) + 2, nx - 1);
-  const int ry0 = max(region_start(qy0, ny), 0), ry1 = min(pidx(qy1 - 1, ny) + 2, ny - 1);
-  const int ox0 = pidx(qx0, nx), ox1 = (qx1 == mx) ? nx : pidx(qx1, nx);
-  const int oy0 = pidx(qy0, ny), oy1 = (qy1 == my) ? ny : pidx(qy1, ny);
-  int t_start = qz0 > 0 ? qz0 - 1 : 0;
-  if (qz0 >= 2 && pidx(qz0, nz) - pidx(qz0 - 1, nz) == 1) t_start = qz0 - 2;
-  const int t_end = min(qz1, mz - 1);
-
-  const TI* __restrict__ in = static_cast<const TI*>(a.in);
-  TD* __restrict__ yout = static_cast<TD*>(a.y);
-  const bool wy = (MODE == 0) && a.write_y;
-  // bounds-checking builds: extents (elements) of the buffers this CTA
-  // addresses; the LVL_* statements below check against them (other builds
-  // run the plain statements)
-#ifdef MGR_DEBUG_BOUNDS
-  const long long n_in = (PK && MODE == 1) ? (long long)nz * a.in_sz - (long long)mz * a.c_sz
-                                           : (long long)(a.in_full ? a.N[0] : nz) * a.in_sz;
-  const long long n_y = PK ? (long long)nz * a.y_sz - (long long)mz * a.c_sz : (long long)a.N[0] * a.y_sz;
-  const long long n_c = (long long)mz * a.c_sz;
-  constexpr long long n_stage = (long long)STAGES * 2 * RR * RC;
-#endif
-#define LVL_CP(dst, src) \
-  MGR_GUARD(MGR_PIN(src, in, n_in, kDbgLevelIn) && MGR_PIN(dst, stage, n_stage, kDbgLevelStage), \
-            cp_async(dst, src, int(sizeof(TI))))
-#define LVL_CPZ(dst, src, valid) \
-  MGR_GUARD(MGR_PIN(src, in, n_in, kDbgLevelIn) && MGR_PIN(dst, stage, n_stage, kDbgLevelStage), \
-            cp_async_zf(dst, src, int(sizeof(TI)), valid))
-#define LVL_Y(q, v) MGR_GUARD(MGR_PIN(q, yout, n_y, kDbgLevelY), *(q) = (v))
-#define LVL_YP(p0, p1, a0, a1, w0, w1, contig)                                                                  \
-  MGR_GUARD((!(w0) || MGR_PIN(p0, yout, n_y, kDbgLevelY)) && (!(w1) || MGR_PIN(p1, yout, n_y, kDbgLevelY)), \
-            store_pair<TD>(p0, p1, a0, a1, w0, w1, contig))
-#define LVL_W(wz, i, v) MGR_GUARD(MGR_IN((wz) - a.w + (i), n_c, kDbgLevelW), (wz)[i] = (v))
-#define LVL_F(i, v) MGR_GUARD(MGR_IN(i, n_c, kDbgLevelF), a.f[i] = (v))
-  const bool afine = AF && MODE == 1 && a.all_fine;
-  const TS qs = QZ ? TS(a.qs) : TS(1);
-  // value written for coefficient v when `st` (the node is stored: values of
-  // nodes that are not stored are never quantized, so never counted as
-  // saturated) (MODE 0); value of a read coefficient (MODE 1)
-  auto yval = [&](TS v, bool st) -> TD {
-    if constexpr (QZ) return st ? TD(quant_code(v, qs, a.qsat)) : TD(0);
-    else return TD(v);
-  };
-  // (MODE 1 with QZ: the code itself; the bin width scales the load vector
-  // once per coarse node instead, see fout)
-  auto cval = [&](TI v) -> TS {
-    if constexpr (QZ && MODE == 1) return code_value<TS>(int(v));
-    else return TS(v);
-  };
-  auto fout = [&](TS acc) -> TW {
-    if constexpr (QZ && MODE == 1) return TW(acc) * TW(a.qs);
-    else return TW(acc);
-  };
-
-  // ---- per-lane column constants (in-plane offsets fit in 32 bits)
-  const int cx0 = 2 * lane;
-  const int gx0 = rx0 + cx0, gx1 = gx0 + 1;
-  const bool vx0 = gx0 <= rx1, vx1 = gx1 <= rx1;
-  const bool fx1 = vx1 && gx1 < nx - 1;  // gx1 is odd: fine unless it is the last node
-  const TS wax1 = fx1 ? a.wa[2][gx1] : TS(0), wbx1 = fx1 ? a.wb[2][gx1] : TS(0);
-  const bool owx0 = vx0 && gx0 >= ox0 && gx0 < ox1, owx1 = vx1 && gx1 >= ox0 && gx1 < ox1;
-  // input columns, clamped into the grid (slots past its end load zeros from a valid address)
-  const int ic0 = a.in_full ? int(fmap(min(gx0, nx - 1), a.s[2], a.N[2])) : min(gx0, nx - 1);
-  const int ic1 = a.in_full ? int(fmap(min(gx1, nx - 1), a.s[2], a.N[2])) : min(gx1, nx - 1);
-  const int yc0 = PK ? gx0 : int(fmap(min(gx0, nx - 1), a.s[2], a.N[2]));
-  const int yc1 = PK ? gx1 : int(fmap(min(gx1, nx - 1), a.s[2], a.N[2]));
-  const bool ycontig = yc1 == yc0 + 1;
-  const int pcx1 = gx1 - cidx(gx1);  // packed column of gx1 in a row coarse in y and z
-
-  // ---- x stencil of this lane's output column
-  const int nbx = qx1 - qx0;
-  const bool kxo = lane < nbx;
-  const int qxo = min(qx0 + lane, mx - 1);
-  const int px = pidx(qxo, nx);
-  const int dx = px - rx0;  // slot of the stencil centre
-  TS kxr[weights_in_smem<TS>() ? 1 : 5];
-  unsigned kxm = 0;  // taps inside the grid
-#pragma unroll
-  for (int o = 0; o < 5; ++o) {
-    const TS kw = a.k[2][5 * qxo + o];
-    if constexpr (weights_in_smem<TS>()) {
-      if (warp == 0) kxs[o * LX + lane] = kw;
-    } else {
-      kxr[o] = kw;
-    }
-    const int j = px + o - 2;
-    if (j >= 0 && j < nx) kxm |= 1u << o;
-  }
-  auto kx = [&](int o) -> TS {
-    if constexpr (weights_in_smem<TS>()) return kxs[o * LX + lane];
-    else return kxr[o];
-  };
-  // interior column: taps px +- 1 fine, px and px +- 2 coarse, even slot
-  const bool kx_generic = kxm == 31u && (px & 1) == 0 && px + 1 < nx - 1;
-  // FP32 (BF): the x / y stencils run without per-row branches, always five
-  // taps (weight 0 outside the grid) over tiles whose slots outside the region
-  // hold zeros, so their 8 independent FMA chains per thread interleave (the
-  // FP32 pass is latency-bound); FP64, bound by its FP64 pipe, keeps the
-  // reduced tap counts of rows whose coefficients vanish.
-  constexpr bool BF = sizeof(TS) == 4;
-  // FP32 nodal decomposition (RS): the coefficients go out after the
-  // coefficient phase, row by row from the shared tile, each lane storing
-  // output columns ox0 + lane and ox0 + LX + lane (consecutive lanes,
-  // consecutive addresses): the coefficient phase then keeps no output
-  // addresses or values live (it is short of registers).  All-coarse nodes
-  // get 0 there, a placeholder a coarser level overwrites.
-  constexpr bool RS = BF && !PK && MODE == 0;
-  const int oc0 = ox0 + lane, oc1 = oc0 + LX;
-  const bool rs0 = oc0 < ox1, rs1 = oc1 < ox1;
-  const int ro0 = int(fmap(min(oc0, nx - 1), a.s[2], a.N[2])), ro1 = int(fmap(min(oc1, nx - 1), a.s[2], a.N[2]));
-  const int rsl0 = oc0 - rx0, rsl1 = oc1 - rx0;
-
-  // ---- per-row constants (RPW row pairs per warp)
-  int gy0[RPW];
-  bool vy0[RPW], vy1[RPW], fy1[RPW], owy0[RPW], owy1[RPW];
-  TS way1[RPW], wby1[RPW];
-  int ir0[RPW], ir1[RPW], yr0[RPW], yr1[RPW];
-  // y stencil of this thread's output rows
-  const int nby = qy1 - qy0;
-  TS kyr[RPW][weights_in_smem<TS>() ? 1 : 5];
-  unsigned kym[RPW];
-  int dyo[RPW];
-#pragma unroll
-  for (int k = 0; k < RPW; ++k) {
-    gy0[k] = ry0 + 2 * (warp * RPW + k);
-    const int g1 = gy0[k] + 1;
-    vy0[k] = gy0[k] <= ry1;
-    vy1[k] = g1 <= ry1;
-    fy1[k] = vy1[k] && g1 < ny - 1;
-    way1[k] = fy1[k] ? a.wa[1][g1] : TS(0);
-    wby1[k] = fy1[k] ? a.wb[1][g1] : TS(0);
-    owy0[k] = vy0[k] && gy0[k] >= oy0 && gy0[k] < oy1;
-    owy1[k] = vy1[k] && g1 >= oy0 && g1 < oy1;
-    const int c0 = min(gy0[k], ny - 1), c1 = min(g1, ny - 1);
-    ir0[k] = int(a.in_full ? fmap(c0, a.s[1], a.N[1]) * a.in_sy : int64_t(c0) * a.in_sy);
-    ir1[k] = int(a.in_full ? fmap(c1, a.s[1], a.N[1]) * a.in_sy : int64_t(c1) * a.in_sy);
-    yr0[k] = PK ? c0 * nx : int(fmap(c0, a.s[1], a.N[1]) * a.y_sy);
-    yr1[k] = PK ? c1 * nx : int(fmap(c1, a.s[1], a.N[1]) * a.y_sy);
-    const int qy = min(qy0 + warp * RPW + k, my - 1);
-    const int py = pidx(qy, ny);
-    dyo[k] = py - ry0;
-    kym[k] = 0;
-#pragma unroll
-    for (int o = 0; o < 5; ++o) {
-      const TS kw = a.k[1][5 * qy + o];
-      if constexpr (weights_in_smem<TS>()) {
-        if (lane == 0) kys[o * (NG * RPW) + warp * RPW + k] = kw;
-      } else {
-        kyr[k][o] = kw;
-      }
-      const int jj = py + o - 2;
-      if (jj >= 0 && jj < ny) kym[k] |= 1u << o;
-    }
-    // rows past the tile's outputs (the last warp's, in all but the last tile
-    // row) are never stored: not interior, so no stencil form reads past the tile
-    if (warp * RPW + k >= nby) kym[k] = 0;
-  }
-  auto ky = [&](int k, int o) -> TS {
-    if constexpr (weights_in_smem<TS>()) return kys[o * (NG * RPW) + warp * RPW + k];
-    else return kyr[k][o];
-  };
-#ifdef MGR_DEBUG_BOUNDS
-  // the shared-tile indices below are a per-thread constant plus the loop's
-  // row and tap offsets: checking the constants' ranges once covers them all
-  (void)MGR_IN(2 * (warp * RPW + RPW - 1) + 1, RR, kDbgLevelTile);  // stage / tile rows
-  (void)MGR_IN(cx0 + 1, RC, kDbgLevelTile);                           // stage / tile columns
-  if (kxo && kx_generic) {
-    (void)MGR_IN(dx - 2, RC, kDbgLevelTile);  // five x taps
-    (void)MGR_IN(dx + 2, RC, kDbgLevelTile);
-  }
-#pragma unroll
-  for (int k = 0; k < RPW; ++k)
-    if (kym[k] == 31u && kxo) {
-      (void)MGR_IN(dyo[k] - 2, RR, kDbgLevelTile);  // five y taps
-      (void)MGR_IN(dyo[k] + 2, RR, kDbgLevelTile);
-    }
-#endif
-  auto iplane = [&](int g) -> int64_t {
-    if (PK && MODE == 1) return int64_t(g) * a.in_sz - int64_t(cidx(g)) * a.c_sz;
-    return a.in_full ? fmap(g, a.s[0], a.N[0]) * a.in_sz : int64_t(g) * a.in_sz;
-  };
-  auto yplane = [&](int g) -> int64_t {
-    return PK ? int64_t(g) * a.y_sz - int64_t(cidx(g)) * a.c_sz : fmap(g, a.s[0], a.N[0]) * a.y_sz;
-  };
-  // ---- plane table, computed once by the CTA (every warp would otherwise
-  // recompute these on each plane pair): plane pair t -- the coarse plane p(t)
-  // and, when a fine plane lies between p(t-1) and p(t), that fine plane -- is
-  // entry t - t_start
-  (void)MGR_IN(t_end - t_start, kLevelPlanes, kDbgLevelTile);
-  for (int e = threadIdx.x; e <= t_end - t_start && e < kLevelPlanes; e += G::NT) {
-    const int t = t_start + e;
-    const int Pc = pidx(t, nz), Pf = Pc - 1;
-    const bool hf = t > t_start && Pc - pidx(t - 1, nz) == 2;
-    ptab[4 * e + 0] = iplane(Pc);
-    ptab[4 * e + 1] = hf ? iplane(Pf) : 0;
-    ptab[4 * e + 2] = yplane(Pc);
-    ptab[4 * e + 3] = yplane(max(Pf, 0));
-    // z stencil weights of both planes for the coarse planes t-1, t, t+1
-    TS* w = pwt + 8 * e;
-#pragma unroll
-    for (int dq = -1; dq <= 1; ++dq) {
-      const int q = t + dq;
-      const bool qv = q >= 0 && q < mz;
-      const int pq = qv ? pidx(q, nz) : 0;
-      const int oc = Pc - pq;
-      w[dq + 1] = (qv && oc >= -2 && oc <= 2) ? a.k[0][5 * q + oc + 2] : TS(0);
-      if (dq < 1) {
-        const int of = Pf - pq;
-        w[dq + 4] = (hf && qv && of >= -2 && of <= 2) ? a.k[0][5 * q + of + 2] : TS(0);
-      }
-    }
-    // z interpolation weights of the fine plane (decomposition)
-    w[6] = (MODE == 0 && hf) ? a.wa[0][Pf] : TS(0);
-    w[7] = (MODE == 0 && hf) ? a.wb[0][Pf] : TS(0);
-    pfl[e] = hf ? 1 : 0;
-  }
-  __syncthreads();  // stencil weights and plane table staged
-  // poff: the plane's offset (plane table); zc: it is a coarse plane (a packed
-  // class then holds only its fine nodes)
-  auto load_plane = [&](TI* sb, int64_t poff, bool zc) {
-    const TI* base = in + poff;
-#pragma unroll
-    for (int k = 0; k < RPW; ++k) {
-      TI* d0 = sb + 2 * (warp * RPW + k) * RC + cx0;
-      if (PK && MODE == 1 && zc) {
-        // rows of a coarse plane: the coarse row gy0 holds its fine columns only
-        const int r0 = ir0[k] - cidx(gy0[k]) * mx, r1 = ir1[k] - cidx(gy0[k] + 1) * mx;
-        if (vy0[k] && fx1) LVL_CP(d0 + 1, base + r0 + pcx1);
-        if (vy1[k]) {
-          if (fy1[k]) {
-            if (vx0) LVL_CP(d0 + RC, base + r1 + ic0);
-            if (vx1) LVL_CP(d0 + RC + 1, base + r1 + ic1);
-          } else if (fx1) {
-            LVL_CP(d0 + RC + 1, base + r1 + pcx1);
-          }
-        }
-        continue;
-      }
-      if constexpr (MODE == 1) {
-        // branch-free: every slot is copied, slots outside the region as zeros
-        // (their addresses are clamped into the grid, so they are valid)
-        LVL_CPZ(d0, base + ir0[k] + ic0, vy0[k] && vx0);
-        LVL_CPZ(d0 + 1, base + ir0[k] + ic1, vy0[k] && vx1);
-        LVL_CPZ(d0 + RC, base + ir1[k] + ic0, vy1[k] && vx0);
-        LVL_CPZ(d0 + RC + 1, base + ir1[k] + ic1, vy1[k] && vx1);
-      } else {
-        // (the decomposition pass is short of registers: copying only the slots
-        // inside the region keeps its per-slot predicates out of the loop)
-        if (vy0[k]) {
-          if (vx0) LVL_CP(d0, base + ir0[k] + ic0);
-          if (vx1) LVL_CP(d0 + 1, base + ir0[k] + ic1);
-        }
-        if (vy1[k]) {
-          if (vx0) LVL_CP(d0 + RC, base + ir1[k] + ic0);
-          if (vx1) LVL_CP(d0 + RC + 1, base + ir1[k] + ic1);
-        }
-      }
-    }
-  };
-  static_assert(STAGES == 1 || STAGES == 2, "one or two stage buffers");
-  // stage buffer of plane pair t (two in rotation, or one)
-  auto stage_of = [&](int t) { return stage + ((STAGES == 2) ? ((t - t_start) & 1) * 2 * RR * RC : 0); };
-  auto issue = [&](int t) {
-    TI* sb = stage_of(t);
-    const int e = t - t_start;
-    const longlong2 off = *reinterpret_cast<const longlong2*>(ptab + 4 * e);
-    load_plane(sb, off.x, true);
-    if (pfl[e]) load_plane(sb + RR * RC, off.y, false);
-    cp_commit();
-  };
-
-  TS Ip[RPW][4], In[RPW][4];
-  TS acc0[RPW], acc1[RPW], acc2[RPW];
-#pragma unroll
-  for (int k = 0; k < RPW; ++k) {
-    acc0[k] = acc1[k] = acc2[k] = TS(0);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) Ip[k][e] = In[k][e] = TS(0);
-  }
-
-  // two stages: the next plane pair is in flight while this one is processed;
-  // one stage: the next is issued once every thread is done with the stage
-  issue(t_start);
-  for (int t = t_start; t <= t_end; ++t) {
-    if (STAGES == 2) {
-      if (t < t_end) {
-        issue(t + 1);  // into the buffer plane pair t-1 used
-        cp_wait<1>();
-      } else {
-        cp_wait<0>();
-      }
-    } else {
-      cp_wait<0>();
-    }
-    // Every thread copies, and later reads, only its own slots of the stage
-    // buffer; the one exception is FP32's read of the next warp's first row
-    // (nxt0 / nxt1 below), which needs the CTA barrier.
-    if constexpr (BF) __syncthreads();
-    else __syncwarp();
-    const TI* sc = stage_of(t);
-    const TI* sf = sc + RR * RC;
-    const int te = t - t_start;
-    const bool hf = pfl[te] != 0;
-    const bool own_c = (t >= qz0) && (t < qz1);
-    const bool own_f = hf && (t > qz0) && (t <= qz1);
-
-    // ---- this thread's values of both planes (pairs from shared memory)
-    TS vc[RPW][4];
-    TI rc[RPW][4];  // raw coarse-plane values: exact copies for the coarse workspace
-#pragma unroll
-    for (int k = 0; k < RPW; ++k) {
-      const int r0 = 2 * (warp * RPW + k);
-      const TI2 p0 = *reinterpret_cast<const TI2*>(sc + r0 * RC + cx0);
-      const TI2 p1 = *reinterpret_cast<const TI2*>(sc + (r0 + 1) * RC + cx0);
-      rc[k][0] = p0.x;
-      rc[k][1] = p0.y;
-      rc[k][2] = p1.x;
-      rc[k][3] = p1.y;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) vc[k][e] = cval(rc[k][e]);
-    }
-    // ---- coarse-z plane: x interpolants of the coarse rows
-    TS v12[RPW];
-#pragma unroll
-    for (int k = 0; k < RPW; ++k) {
-      const TS v02 = __shfl_down_sync(FULL, vc[k][0], 1, LX);
-      v12[k] = __shfl_down_sync(FULL, vc[k][2], 1, LX);
-      if (MODE == 0) {
-        In[k][0] = vc[k][0];
-        In[k][1] = fx1 ? wax1 * vc[k][0] + wbx1 * v02 : vc[k][1];
-      }
-    }
-    // the x interpolant of the coarse row below this warp's last pair (the next
-    // warp's first row), for the y interpolation of this warp's last fine row.
-    // FP32: computed here from the staged tile (the same operations as the next
-    // warp's), so no exchange and no barrier is needed; FP64, bound by its FP64
-    // pipe, takes it from the next warp through shared memory instead.
-    TS nxt0 = TS(0), nxt1 = TS(0);
-    if constexpr (!BF) {
-      if (MODE == 0) *reinterpret_cast<TS2*>(xch + warp * RC + cx0) = TS2{In[0][0], In[0][1]};
-      __syncthreads();
-    } else if (MODE == 0 && (LX < 32 || warp + 1 < NG)) {
-      // (half-warp groups: both halves of a warp take this branch, so that the
-      // shuffle below runs on every lane; the last group's result is unused)
-      const int wn = LX < 32 ? min(warp + 1, NG - 1) : warp + 1;
-      const TI2 pn = *reinterpret_cast<const TI2*>(sc + 2 * wn * RPW * RC + cx0);
-      const TS vn0 = cval(pn.x), vn1 = cval(pn.y);
-      const TS vn2 = __shfl_down_sync(FULL, vn0, 1, LX);
-      nxt0 = vn0;
-      nxt1 = fx1 ? wax1 * vn0 + wbx1 * vn2 : vn1;
-    }
-
-    // ---- coefficients of both planes -> shared memory and the nodal output
-    TS* cc = cbuf;
-    TS* cf = cbuf + RR * CP;
-    const longlong2 yoff = *reinterpret_cast<const longlong2*>(ptab + 4 * te + 2);
-    TD* yzc = yout + yoff.x;
-    TD* yzf = yout + yoff.y;
-#pragma unroll
-    for (int k = 0; k < RPW; ++k) {
-      const int r0 = 2 * (warp * RPW + k);
-      TS c[4];
-      if (MODE == 0) {
-        TS n0, n1;
-        if (k + 1 < RPW) {
-          n0 = In[k + 1 < RPW ? k + 1 : k][0];
-          n1 = In[k + 1 < RPW ? k + 1 : k][1];
-        } else if (warp + 1 < NG) {
-          if constexpr (BF) {
-            n0 = nxt0;
-            n1 = nxt1;
-          } else {
-            const TS2 nx2 = *reinterpret_cast<const TS2*>(xch + (warp + 1) * RC + cx0);
-            n0 = nx2.x;
-            n1 = nx2.y;
-          }
-        } else {
-          n0 = n1 = TS(0);
-        }
-        if (fy1[k]) {
-          In[k][2] = way1[k] * In[k][0] + wby1[k] * n0;
-          In[k][3] = way1[k] * In[k][1] + wby1[k] * n1;
-        } else {
-          In[k][2] = vc[k][2];
-          In[k][3] = fx1 ? wax1 * vc[k][2] + wbx1 * v12[k] : vc[k][3];
-        }
-        c[0] = TS(0);
-        c[1] = vc[k][1] - In[k][1];
-        c[2] = vc[k][2] - In[k][2];
-        c[3] = vc[k][3] - In[k][3];
-      } else if (afine) {
-        c[0] = (vx0 && vy0[k]) ? vc[k][0] : TS(0);
-        c[1] = (vx1 && vy0[k]) ? vc[k][1] : TS(0);
-        c[2] = (vx0 && vy1[k]) ? vc[k][2] : TS(0);
-        c[3] = (vx1 && vy1[k]) ? vc[k][3] : TS(0);
-      } else {
-        c[0] = TS(0);
-        c[1] = fx1 ? vc[k][1] : TS(0);
-        c[2] = fy1[k] ? vc[k][2] : TS(0);
-        c[3] = (fx1 || fy1[k]) ? vc[k][3] : TS(0);
-      }
-      if constexpr (BF && (PK || MODE == 0)) {
-        // slots outside the region hold zeros, not values of unloaded slots (the
-        // nodal recomposition loads zero-fill them; the other loads skip them)
-        c[0] = (vx0 && vy0[k]) ? c[0] : TS(0);
-        c[1] = (vx1 && vy0[k]) ? c[1] : TS(0);
-        c[2] = (vx0 && vy1[k]) ? c[2] : TS(0);
-        c[3] = (vx1 && vy1[k]) ? c[3] : TS(0);
-      }
-      if constexpr (!BF) {
-        *reinterpret_cast<TS2*>(cc + r0 * CP + cx0) = TS2{c[0], c[1]};
-        *reinterpret_cast<TS2*>(cc + (r0 + 1) * CP + cx0) = TS2{c[2], c[3]};
-      }
-      TS dd[4] = {TS(0), TS(0), TS(0), TS(0)};  // fine-plane coefficients (zeros without a fine plane)
-      if (PK && wy && own_c) {
-        // packed class: the coarse row gy0 keeps only its fine column gx1
-        const int r0 = yr0[k] - cidx(gy0[k]) * mx, r1 = yr1[k] - cidx(gy0[k] + 1) * mx;
-        if (owy0[k] && owx1 && fx1) LVL_Y(yzc + r0 + pcx1, yval(c[1], true));
-        if (owy1[k]) {
-          if (fy1[k]) {
-            LVL_YP(yzc + r1 + yc0, yzc + r1 + yc1, yval(c[2], owx0), yval(c[3], owx1), owx0, owx1, true);
-          } else if (owx1 && fx1) {
-            LVL_Y(yzc + r1 + pcx1, yval(c[3], true));
-          }
-        }
-      } else if (!RS && wy && own_c) {
-        // all-coarse nodes get their (uncorrected) value as a placeholder that a
-        // coarser level overwrites; it keeps the row's sectors fully written
-        LVL_YP(yzc + yr0[k] + yc0, yzc + yr0[k] + yc1, TD(vc[k][0]), TD(fx1 ? c[1] : vc[k][1]),
-                       owy0[k] && owx0, owy0[k] && owx1, ycontig);
-        LVL_YP(yzc + yr1[k] + yc0, yzc + yr1[k] + yc1, TD(fy1[k] ? c[2] : vc[k][2]),
-                       TD((fx1 || fy1[k]) ? c[3] : vc[k][3]), owy1[k] && owx0, owy1[k] && owx1, ycontig);
-      }
-      if (MODE == 0 && own_c) {
-        // coarse nodal values of the owned all-coarse nodes
-        TW* wz = a.w + int64_t(t) * a.c_sz;
-        if (owy0[k] && owx0) LVL_W(wz, int64_t(cidx(gy0[k])) * a.c_sy + cidx(gx0), TW(rc[k][0]));
-        if (owy0[k] && owx1 && !fx1) LVL_W(wz, int64_t(cidx(gy0[k])) * a.c_sy + cidx(gx1), TW(rc[k][1]));
-        if (owy1[k] && !fy1[k]) {
-          if (owx0) LVL_W(wz, int64_t(cidx(gy0[k] + 1)) * a.c_sy + cidx(gx0), TW(rc[k][2]));
-          if (owx1 && !fx1) LVL_W(wz, int64_t(cidx(gy0[k] + 1)) * a.c_sy + cidx(gx1), TW(rc[k][3]));
-        }
-      }
-      if (hf) {
-        TS vf[4];
-        {
-          const TI2 f0 = *reinterpret_cast<const TI2*>(sf + r0 * RC + cx0);
-          const TI2 f1 = *reinterpret_cast<const TI2*>(sf + (r0 + 1) * RC + cx0);
-          vf[0] = cval(f0.x);
-          vf[1] = cval(f0.y);
-          vf[2] = cval(f1.x);
-          vf[3] = cval(f1.y);
-        }
-        TS d[4];
-        if (MODE == 0) {
-          const TS za = pwt[8 * te + 6], zb = pwt[8 * te + 7];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) d[e] = vf[e] - za * Ip[k][e] - zb * In[k][e];
-        } else {
-#pragma unroll
-          for (int e = 0; e < 4; ++e) d[e] = vf[e];
-        }
-        if constexpr (BF && (PK || MODE == 0)) {
-          d[0] = (vx0 && vy0[k]) ? d[0] : TS(0);
-          d[1] = (vx1 && vy0[k]) ? d[1] : TS(0);
-          d[2] = (vx0 && vy1[k]) ? d[2] : TS(0);
-          d[3] = (vx1 && vy1[k]) ? d[3] : TS(0);
-        }
-        if constexpr (!BF) {
-          *reinterpret_cast<TS2*>(cf + r0 * CP + cx0) = TS2{d[0], d[1]};
-          *reinterpret_cast<TS2*>(cf + (r0 + 1) * CP + cx0) = TS2{d[2], d[3]};
-        }
-#pragma unroll
-        for (int e = 0; e < 4; ++e) dd[e] = d[e];
-        if (!RS && wy && own_f) {
-          LVL_YP(yzf + yr0[k] + yc0, yzf + yr0[k] + yc1, yval(d[0], owy0[k] && owx0), yval(d[1], owy0[k] && owx1), owy0[k] && owx0,
-                         owy0[k] && owx1, ycontig);
-          LVL_YP(yzf + yr1[k] + yc0, yzf + yr1[k] + yc1, yval(d[2], owy1[k] && owx0), yval(d[3], owy1[k] && owx1), owy1[k] && owx0,
-                         owy1[k] && owx1, ycontig);
-        }
-      }
-      if constexpr (BF) {
-        // FP32: both planes interleaved, {coarse plane, fine plane} per node
-        *reinterpret_cast<float4*>(cbuf + 2 * (r0 * CP + cx0)) = make_float4(c[0], dd[0], c[1], dd[1]);
-        *reinterpret_cast<float4*>(cbuf + 2 * ((r0 + 1) * CP + cx0)) = make_float4(c[2], dd[2], c[3], dd[3]);
-      }
-    }
-    // The x stencil and the row stores read only this warp's rows of the
-    // coefficient tile: a warp barrier orders them.  With one stage buffer,
-    // FP32 reloads the buffer whose rows the warp above still reads (nxt0 /
-    // nxt1): a CTA barrier then.  (The x-stencil results that the y stencil
-    // reads across warps are written after the previous plane pair's last CTA
-    // barrier and read after this one's.)
-    if constexpr (BF && STAGES == 1) __syncthreads();
-    else __syncwarp();
-
-    if (STAGES == 1 && t < t_end) issue(t + 1);  // every thread is done with the stage buffer
-
-    // ---- coefficients of this warp's owned rows (RS), from the shared tile
-    if constexpr (RS) {
-      if (wy && (own_c || own_f)) {
-#pragma unroll
-        for (int k = 0; k < RPW; ++k) {
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int r = 2 * (warp * RPW + k) + h;
-            const bool orow = h == 0 ? owy0[k] : owy1[k];
-            const int yr = h == 0 ? yr0[k] : yr1[k];
-            // {coarse plane, fine plane} pairs of the interleaved tile
-            const float2 v0 = *reinterpret_cast<const float2*>(cbuf + 2 * (r * CP + rsl0));
-            const float2 v1 = *reinterpret_cast<const float2*>(cbuf + 2 * (r * CP + rsl1));
-            if (orow && own_c) {
-              if (rs0) LVL_Y(yzc + yr + ro0, TD(v0.x));
-              if (rs1) LVL_Y(yzc + yr + ro1, TD(v1.x));
-            }
-            if (orow && own_f) {
-              if (rs0) LVL_Y(yzf + yr + ro0, TD(v0.y));
-              if (rs1) LVL_Y(yzf + yr + ro1, TD(v1.y));
-            }
-          }
-        }
-      }
-    }
-
-    // ---- x stencil on every row of this warp (both planes)
-    if constexpr (BF) {
-      // FP32, both planes at once: {coarse, fine} pairs in the interleaved
-      // tiles, paired FMAs (the results equal two scalar FMA chains)
-      if (kxo && kx_generic) {
-        // every row's five taps from two 16-byte loads and one 8-byte load
-#pragma unroll
-        for (int k = 0; k < RPW; ++k) {
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int r = 2 * (warp * RPW + k) + h;
-            const float* row = cbuf + 2 * (r * CP + dx - 2);
-            const float4 t01 = *reinterpret_cast<const float4*>(row);
-            const float4 t23 = *reinterpret_cast<const float4*>(row + 4);
-            const float2 t4 = *reinterpret_cast<const float2*>(row + 8);
-            float2 g = __fmul2_rn(make_float2(kx(0), kx(0)), make_float2(t01.x, t01.y));
-            g = __ffma2_rn(make_float2(kx(1), kx(1)), make_float2(t01.z, t01.w), g);
-            g = __ffma2_rn(make_float2(kx(2), kx(2)), make_float2(t23.x, t23.y), g);
-            g = __ffma2_rn(make_float2(kx(3), kx(3)), make_float2(t23.z, t23.w), g);
-            g = __ffma2_rn(make_float2(kx(4), kx(4)), t4, g);
-            *reinterpret_cast<float2*>(gxb + 2 * (r * GP + lane)) = g;
-          }
-        }
-      } else if (kxo) {
-        // boundary columns: clamped slots, weight 0 outside the grid
-#pragma unroll
-        for (int k = 0; k < RPW; ++k) {
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int r = 2 * (warp * RPW + k) + h;
-            float2 g = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int o = 0; o < 5; ++o) {
-              const int j = min(max(dx - 2 + o, 0), RC - 1);  // weight 0 where clamped
-              g = __ffma2_rn(make_float2(kx(o), kx(o)), *reinterpret_cast<const float2*>(cbuf + 2 * (r * CP + j)), g);
-            }
-            *reinterpret_cast<float2*>(gxb + 2 * (r * GP + lane)) = g;
-          }
-        }
-      }
-    } else if (kxo) {
-#pragma unroll
-      for (int k = 0; k < RPW; ++k) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int r = 2 * (warp * RPW + k) + h;
-          // rows coarse in y (of the coarse-z plane): c vanishes on coarse columns
-          const bool zero_row = (h == 0 || !fy1[k]) && !afine;
-          TS g, gf = TS(0);
-          if (kx_generic) {
-            const TS* row = cc + r * CP + dx - 2;
-            const TS2 a01 = *reinterpret_cast<const TS2*>(row);
-            const TS2 a23 = *reinterpret_cast<const TS2*>(row + 2);
-            if (zero_row) {
-              g = kx(1) * a01.y + kx(3) * a23.y;
-            } else {
-              g = kx(0) * a01.x + kx(1) * a01.y + kx(2) * a23.x + kx(3) * a23.y + kx(4) * row[4];
-            }
-            if (hf) {
-              const TS* rf = cf + r * CP + dx - 2;
-              const TS2 b01 = *reinterpret_cast<const TS2*>(rf);
-              const TS2 b23 = *reinterpret_cast<const TS2*>(rf + 2);
-              gf = kx(0) * b01.x + kx(1) * b01.y + kx(2) * b23.x + kx(3) * b23.y + kx(4) * rf[4];
-            }
-          } else {
-            g = TS(0);
-#pragma unroll
-            for (int o = 0; o < 5; ++o)
-              if (kxm & (1u << o)) {
-                g += kx(o) * cc[r * CP + dx - 2 + o];
-                if (hf) gf += kx(o) * cf[r * CP + dx - 2 + o];
-              }
-          }
-          gxb[r * GP + lane] = g;
-          if (hf) gxb[RR * GP + r * GP + lane] = gf;
-        }
-      }
-    }
-    __syncthreads();
-
-    // ---- y stencil and z accumulation for this thread's outputs
-    // z weights of the two planes for coarse planes t-1, t, t+1 (plane table)
-    TS wzc[3], wzf[2];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) wzc[i] = pwt[8 * te + i];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) wzf[i] = pwt[8 * te + 3 + i];
-#pragma unroll
-    for (int k = 0; k < RPW; ++k) {
-      const int j = warp * RPW + k;
-      if constexpr (BF) {
-        // both planes at once ({coarse, fine} pairs, paired FMAs), five taps;
-        // rows clamped into the tile (weight 0 where clamped); computed on
-        // every lane of a row slot with outputs (j < nby: uniform across the
-        // row group), stored only where the output exists
-        if (j < nby) {
-          const float* gcol = gxb + 2 * lane;
-          float2 g;
-          if (kym[k] == 31u) {
-            const float* g0 = gcol + 2 * (dyo[k] - 2) * GP;
-            g = __fmul2_rn(make_float2(ky(k, 0), ky(k, 0)), *reinterpret_cast<const float2*>(g0));
-#pragma unroll
-            for (int o = 1; o < 5; ++o)
-              g = __ffma2_rn(make_float2(ky(k, o), ky(k, o)), *reinterpret_cast<const float2*>(g0 + 2 * o * GP), g);
-          } else {
-            g = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int o = 0; o < 5; ++o) {
-              const int rr = min(max(dyo[k] + o - 2, 0), RR - 1);
-              g = __ffma2_rn(make_float2(ky(k, o), ky(k, o)), *reinterpret_cast<const float2*>(gcol + 2 * rr * GP), g);
-            }
-          }
-          const TS gc = g.x, gf = g.y;
-          acc0[k] += wzc[0] * gc;
-          acc1[k] += wzc[1] * gc;
-          acc2[k] += wzc[2] * gc;
-          acc0[k] += wzf[0] * gf;
-          acc1[k] += wzf[1] * gf;
-          if (kxo && t - 1 >= qz0 && t - 1 < qz1)
-            LVL_F(int64_t(t - 1) * a.c_sz + int64_t(qy0 + j) * a.c_sy + qxo, fout(acc0[k]));
-        }
-      } else if (j < nby && kxo) {
-        TS gc = TS(0), gf = TS(0);
-        const TS* gcol = gxb + (dyo[k] - 2) * GP + lane;
-        if (kym[k] == 31u) {  // interior row: all five taps inside the grid
-          gc = ky(k, 0) * gcol[0] + ky(k, 1) * gcol[GP] + ky(k, 2) * gcol[2 * GP] + ky(k, 3) * gcol[3 * GP] +
-               ky(k, 4) * gcol[4 * GP];
-          if (hf) {
-            const TS* fcol = gcol + RR * GP;
-            gf = ky(k, 0) * fcol[0] + ky(k, 1) * fcol[GP] + ky(k, 2) * fcol[2 * GP] + ky(k, 3) * fcol[3 * GP] +
-                 ky(k, 4) * fcol[4 * GP];
-          }
-        } else {
-#pragma unroll
-          for (int o = 0; o < 5; ++o) {
-            if (kym[k] & (1u << o)) {
-              gc += ky(k, o) * gxb[(dyo[k] + o - 2) * GP + lane];
-              if (hf) gf += ky(k, o) * gxb[RR * GP + (dyo[k] + o - 2) * GP + lane];
-            }
-          }
-        }
-        acc0[k] += wzc[0] * gc;
-        acc1[k] += wzc[1] * gc;
-        acc2[k] += wzc[2] * gc;
-        if (hf) {
-          acc0[k] += wzf[0] * gf;
-          acc1[k] += wzf[1] * gf;
-        }
-        if (t - 1 >= qz0 && t - 1 < qz1)
-          LVL_F(int64_t(t - 1) * a.c_sz + int64_t(qy0 + j) * a.c_sy + qxo, fout(acc0[k]));
-      }
-      acc0[k] = acc1[k];
-      acc1[k] = acc2[k];
-      acc2[k] = TS(0);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) Ip[k][e] = In[k][e];
-    }
-  }
-  if (t_end == mz - 1 && qz1 == mz) {
-#pragma unroll
-    for (int k = 0; k < RPW; ++k) {
-      const int j = warp * RPW + k;
-      if (j < nby && kxo) LVL_F(int64_t(mz - 1) * a.c_sz + int64_t(qy0 + j) * a.c_sy + qxo, fout(acc0[k]));
-    }
-  }
-}
-
-#undef LVL_CP
-#undef LVL_CPZ
-#undef LVL_Y
-#undef LVL_YP
-#undef LVL_W
-#undef LVL_F
-
-template <int MODE, int NW, int RPW, int STAGES, typename TI, typename TD, typename TS, typename TW, bool PK, bool QZ>
-__global__ void __launch_bounds__(NW * 32, level_ctas_per_sm(NW)) k_level(const LevelArgs<TS, TW> a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  level_body<MODE, NW, RPW, STAGES, TI, TD, TS, TW, PK, QZ>(a, blockIdx.x, blockIdx.y, blockIdx.z + a.bz0, smem_raw);
 }
 
 // ---------------------------------------------------------------------------

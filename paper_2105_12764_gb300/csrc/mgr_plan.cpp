@@ -138,11 +138,13 @@ int build_plan_tables(mgr_plan* p) {
       ax.o_wa = push(n);
       ax.o_wb = push(n);
       ax.o_k = push(size_t(5) * m);
+      ax.o_slot = push(size_t(kSlot) * m);
       ax.o_ta = push(m);
       ax.o_tb = push(m);
       if (!ax.active) {
         // identity stencil, no solve
         T[ax.o_k + 2] = 1.0;
+        T[ax.o_slot + 2] = 1.0;
         continue;
       }
       // level-l coordinates
@@ -211,6 +213,22 @@ int build_plan_tables(mgr_plan* p) {
         for (int t = 0; t < 5; ++t) T[ax.o_k + 5 * q + t] = K[size_t(5) * q + t] * inv;
         T[ax.o_ta + q] = q > 0 ? ce[q - 1] * inv : 0.0;
         T[ax.o_tb + q] = q < m - 1 ? ce[q] * inv : 0.0;
+      }
+      // the same rows by slots: with n even the last two nodes are both coarse,
+      // so node m-2's right neighbour and node m-1's left neighbour are coarse
+      for (int q = 0; q < m; ++q) {
+        const double* k = &T[ax.o_k + 5 * q];
+        double* s = &T[ax.o_slot + int64_t(kSlot) * q];
+        const bool even = n % 2 == 0;
+        s[0] = even && q == m - 1 ? k[1] : k[0];
+        s[1] = even && q == m - 1 ? 0.0 : k[1];
+        s[2] = k[2];
+        s[3] = even && q == m - 2 ? 0.0 : k[3];
+        s[4] = even && q == m - 2 ? k[3] : k[4];
+        if (2 * q + 1 < n - 1) {
+          s[5] = T[ax.o_wa + 2 * q + 1];
+          s[6] = T[ax.o_wb + 2 * q + 1];
+        }
       }
     }
   }

@@ -41,6 +41,7 @@
 #include <algorithm>
 #include <cstdint>
 #include <cstdio>
+#include <type_traits>
 
 #include "mgr_internal.h"
 
@@ -56,6 +57,7 @@ namespace {
 // slice j is the level time index t = min(first + j * step, last).
 struct Slabs {
   int zchunks;
+  int base = 0;              // first slice of this launch (level pass)
   int first, step, last;
   int nt;                    // level time length n_t
   int64_t tS, tN;            // full-grid time map: index min(t * tS, tN - 1)
@@ -70,10 +72,10 @@ __device__ __forceinline__ int64_t slab_map(const Slabs& sl, int t, int full) {
   return full ? fmap(t, sl.tS, sl.tN) : int64_t(t);
 }
 
-template <int MODE, int NW, int RPW, int STAGES, typename TI, typename TD, typename TS, typename TW>
-__global__ void __launch_bounds__(NW * 32, level_ctas_per_sm(NW)) k_level_st(const LevelArgs<TS, TW> a, const Slabs sl) {
+template <int MODE, typename TI, typename TD, typename TS, typename TW, bool S1>
+__global__ void __launch_bounds__(32, level_ctas<MODE, TS>()) k_level_st(const LevelArgs<TS, TW> a, const Slabs sl) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int j = blockIdx.z / sl.zchunks, bz = blockIdx.z - j * sl.zchunks;
+  const int js = blockIdx.y / sl.zchunks, bz = blockIdx.y - js * sl.zchunks, j = sl.base + js;
   const int t = slab_time(sl, j);
   LevelArgs<TS, TW> b = a;
   b.in = static_cast<const TI*>(a.in) + slab_map(sl, t, sl.in_tfull) * sl.in_ts;
@@ -83,7 +85,7 @@ __global__ void __launch_bounds__(NW * 32, level_ctas_per_sm(NW)) k_level_st(con
   }
   b.f = a.f + int64_t(t) * sl.f_ts;
   b.all_fine = (MODE == 1 && sl.fine_all) ? int(!is_coarse(t, sl.nt)) : 0;
-  level_body<MODE, NW, RPW, STAGES, TI, TD, TS, TW, false, false, true>(b, blockIdx.x, blockIdx.y, bz, smem_raw);
+  level_body<MODE, TI, TD, TS, TW, S1, false, false, true>(b, blockIdx.x, bz, smem_raw);
 }
 
 template <int NW, int RPW, typename TD, typename TO, typename TS, typename TW>
@@ -213,16 +215,19 @@ Slabs base_slabs(const mgr_plan* p, int l) {
 template <int MODE, typename TI, typename TD, typename TS, typename TW>
 cudaError_t launch_level_st(const mgr_plan* p, LevelArgs<TS, TW>& a, Slabs sl, int slabs, cudaStream_t st) {
   if (slabs <= 0) return cudaSuccess;
-  using C = LevelCfg<TS>;
-  using G = LevelTile<C::NW, C::RPW>;
-  constexpr size_t sm = level_smem_bytes<C::NW, C::RPW, C::STAGES, TI, TS>();
-  const int gx = (a.m[2] + G::BX - 1) / G::BX, gy = (a.m[1] + G::BY - 1) / G::BY;
-  const int chunks = choose_chunks(p, int64_t(gx) * gy * slabs, a.m[0], level_ctas_per_sm(C::NW), kLevelMaxChunk);
-  a.qz_chunk = (a.m[0] + chunks - 1) / chunks;
+  level_shape<MODE, TI, false>(p, a, slabs);
   sl.zchunks = (a.m[0] + a.qz_chunk - 1) / a.qz_chunk;
-  auto kern = k_level_st<MODE, C::NW, C::RPW, C::STAGES, TI, TD, TS, TW>;
+  const size_t sm = level_smem_bytes<MODE, TI, TS>(a.rows, level_slot_rows(a.m[2], a.m[1], a.rows));
+  auto kern = a.s[2] == 1 ? k_level_st<MODE, TI, TD, TS, TW, true> : k_level_st<MODE, TI, TD, TS, TW, false>;
   raise_smem_limit(kern, sm);
-  kern<<<dim3(gx, gy, sl.zchunks * slabs), C::NW * 32, sm, st>>>(a, sl);
+  // slices in groups: the grid's y extent is limited to 65535
+  const int per = std::max(1, 65535 / sl.zchunks);
+  for (int s0 = 0; s0 < slabs; s0 += per) {
+    Slabs part = sl;
+    part.base = s0;
+    kern<<<dim3(unsigned(level_warps<32>(a.m[2], a.m[1], a.rows)), sl.zchunks * std::min(per, slabs - s0)), 32, sm, st>>>(
+        a, part);
+  }
   return cudaGetLastError();
 }
 
@@ -369,7 +374,6 @@ cudaError_t decompose_st_t(const mgr_plan* p, const void* in, void* out, void* w
       rec_begin(st);
       if (l == L) {
         a.in = in;
-        a.in_full = 1;
         a.in_sz = p->full[1] * p->full[2];
         a.in_sy = p->full[2];
         sl.in_tfull = 1;
@@ -377,7 +381,6 @@ cudaError_t decompose_st_t(const mgr_plan* p, const void* in, void* out, void* w
         e = launch_level_st<0, TD, TD, TS, TW>(p, a, sl, mt, st);
       } else {
         a.in = cur;
-        a.in_full = 0;
         a.in_sz = int64_t(g.ax[1].n) * g.ax[2].n;
         a.in_sy = g.ax[2].n;
         sl.in_tfull = 0;
@@ -401,7 +404,6 @@ cudaError_t decompose_st_t(const mgr_plan* p, const void* in, void* out, void* w
     {
       auto a = level_args<TS, TW>(p, l);
       a.in = out;
-      a.in_full = 1;
       a.in_sz = p->full[1] * p->full[2];
       a.in_sy = p->full[2];
       a.f = G;
@@ -454,7 +456,6 @@ cudaError_t recompose_st_t(const mgr_plan* p, const void* in, void* out, void* w
     {
       auto a = level_args<TS, TW>(p, l);
       a.in = in;
-      a.in_full = 1;
       a.in_sz = p->full[1] * p->full[2];
       a.in_sy = p->full[2];
       a.f = G;
