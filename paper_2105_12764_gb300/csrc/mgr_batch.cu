@@ -77,17 +77,17 @@ __global__ void __launch_bounds__(32, level_ctas<MODE, TS>()) kb_level(const Lev
   }
 }
 
-template <int NW, int RPW, typename TD, typename TO, typename TS, typename TW, int LX = 32>
-__global__ void __launch_bounds__(NW * 32, level_ctas_per_sm(NW)) kb_interp(const InterpArgs<TS, TW>* __restrict__ args,
-                                                        const int4* __restrict__ items, int n) {
+template <typename TD, typename TO, typename TS, typename TW, bool S1>
+__global__ void __launch_bounds__(32, 16) kb_interp(const InterpArgs<TS, TW>* __restrict__ args,
+                                                    const int4* __restrict__ items, int n) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(16) InterpArgs<TS, TW> sa;
   for (int i = blockIdx.x; i < n; i += gridDim.x) {
     const int4 it = items[i];
     copy_words(&sa, args + it.x);
-    __syncthreads();
-    interp_body<NW, RPW, TD, TO, TS, TW, false, false, LX>(sa, it.y, it.z, it.w, smem_raw);
-    __syncthreads();
+    __syncwarp();
+    interp_body<TD, TO, TS, TW, S1>(sa, it.y, it.w, smem_raw);
+    __syncwarp();
   }
 }
 
@@ -226,7 +226,6 @@ inline const char* cfg_name(int cfg) { return cfg == 0 ? "30x14" : cfg == 1 ? "3
 #ifndef MGR_BATCH_CHUNK_MAX
 #define MGR_BATCH_CHUNK_MAX 32
 #endif
-static_assert(MGR_BATCH_CHUNK_MAX <= kLevelMaxChunk, "interpolation chunks are at most kLevelMaxChunk planes");
 #if MGR_BATCH_CHUNK_MAX > 32
 constexpr int kChunks[] = {8, 16, 32, MGR_BATCH_CHUNK_MAX};
 #else
@@ -236,6 +235,9 @@ constexpr int kChunks[] = {8, 16, 32};
 // Resident one-warp level-pass CTAs per SM a persistent launch asks for (the
 // shared memory of 14-row strips allows 18 in FP32).
 constexpr int kLevelResident = 16;
+
+// Coarse rows per interpolation strip, at most (split evenly over a field's strips).
+constexpr int kInterpRows = 4;
 
 // Coarse z planes per work item: at most `chunk`, split evenly over the items
 // (33 planes in chunks of 32 are 17 + 16, not 32 + 1).
@@ -390,15 +392,7 @@ struct Builder {
   void interp_phase(int d) {
     std::vector<InterpArgs<TS, TW>> descs;
     std::vector<int4> items;
-#ifndef MGR_BATCH_INTERP_NW
-#define MGR_BATCH_INTERP_NW 1
-#endif
-#ifndef MGR_BATCH_INTERP_LX
-#define MGR_BATCH_INTERP_LX 16
-#endif
-    // tiles of LX x BY coarse nodes: half-warp row groups fit the short coarse
-    // rows of the batch's fields better than whole warps
-    constexpr int NW = MGR_BATCH_INTERP_NW, RPW = 2, LX = MGR_BATCH_INTERP_LX, BY = NW * 32 / LX * RPW;
+    size_t smem = 0;  // the largest item's
     for (size_t fi = 0; fi < fields.size(); ++fi) {
       const FieldRef& fr = fields[fi];
       const int L = fr.p->levels;
@@ -413,8 +407,7 @@ struct Builder {
         a.m[k] = g.ax[k].m;
         a.s[k] = g.ax[k].s;
         a.N[k] = g.ax[k].N;
-        a.wa[k] = T + g.ax[k].o_wa;
-        a.wb[k] = T + g.ax[k].o_wb;
+        a.slot[k] = T + g.ax[k].o_slot;
       }
       // the coarse values of level l-1 and the level-l destination
       char* cur = ((L - l) % 2 == 0) ? bufA(fr) : bufB(fr);
@@ -427,16 +420,16 @@ struct Builder {
       a.c_sy = g.ax[2].m;
       const bool last = (l == L);
       a.out = last ? fr.out : static_cast<void*>(nxt);
-      a.out_full = last ? 1 : 0;
       a.o_sz = last ? a.y_sz : int64_t(g.ax[1].n) * g.ax[2].n;
       a.o_sy = last ? a.y_sy : int64_t(g.ax[2].n);
+      a.rows = balanced_chunk(kInterpRows, g.ax[1].m);
       a.qz_chunk = balanced_chunk(cand.chunk, g.ax[0].m);
       const int di = int(descs.size());
       descs.push_back(a);
-      const int gx = (a.m[2] + LX - 1) / LX, gy = (a.m[1] + BY - 1) / BY, gz = (a.m[0] + a.qz_chunk - 1) / a.qz_chunk;
+      smem = std::max(smem, interp_smem_bytes<TD, TS, TW>(a.rows, level_slot_rows(a.m[2], a.m[1], a.rows)));
+      const int gx = int(interp_warps(a.m[2], a.m[1], a.rows)), gz = (a.m[0] + a.qz_chunk - 1) / a.qz_chunk;
       for (int z = 0; z < gz; ++z)
-        for (int y = 0; y < gy; ++y)
-          for (int x = 0; x < gx; ++x) items.push_back(make_int4(di, x, y, z));
+        for (int x = 0; x < gx; ++x) items.push_back(make_int4(di, x, 0, z));
     }
     if (items.empty()) return;
     PendingPhase ph{};
@@ -444,10 +437,11 @@ struct Builder {
     ph.desc_off = blob.put(descs.data(), descs.size() * sizeof(descs[0]));
     ph.items_off = blob.put(items.data(), items.size() * sizeof(int4));
     ph.n_items = int(items.size());
-    ph.fn = reinterpret_cast<const void*>(kb_interp<NW, RPW, TD, TO, TS, TW, LX>);
-    ph.block = NW * 32;
-    ph.smem = interp_smem_bytes<NW, RPW, TD, TS, TW, LX>();
-    ph.grid = std::min(ph.n_items, num_sms * level_ctas_per_sm(NW));
+    ph.fn = d == 0 ? reinterpret_cast<const void*>(kb_interp<TD, TO, TS, TW, true>)
+                   : reinterpret_cast<const void*>(kb_interp<TD, TO, TS, TW, false>);
+    ph.block = 32;
+    ph.smem = smem;
+    ph.grid = std::min(ph.n_items, num_sms * 16);
     pending.push_back(ph);
   }
 

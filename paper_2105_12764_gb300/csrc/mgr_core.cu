@@ -428,7 +428,8 @@ cudaError_t recompose_t(const mgr_plan* p, const void* in, void* out, void* ws, 
     rec_begin(st);
     if (l == L && rp) {
       for (int k = 0; k < rp->iparts; ++k) {
-        launch_interp_chunks<TY, TD, TS, TW, PK, QZ>(p, l, cl, cur, out, 1, st, qs, rp->ic0[k], rp->ic0[k + 1]);
+        launch_interp_chunks<TY, TD, TS, TW, PK, QZ>(p, l, cl, cur, out, 1, st, qs, rp->ic0[k], rp->ic0[k + 1],
+                                                     pipe_planes(g.ax[0].m));
         if (cudaEventRecord(rp->done[k], st) != cudaSuccess) return cudaGetLastError();
       }
     } else if (l == L) {
@@ -535,9 +536,9 @@ cudaError_t host_rec_pipe_t(const mgr_plan* p, const void* host_in, void* host_o
   const int parts = std::min(gz, kPipeParts);
   int c0[kPipeParts + 1];
   for (int k = 0; k <= parts; ++k) c0[k] = int((int64_t(k) * gz) / parts);
-  int gx, gy;
-  auto ia = interp_args<TS, TW, false>(p, L, nullptr, nullptr, nullptr, 1, 1.0, &gx, &gy);
-  const int giz = interp_chunks(p, ia, gx, gy), iqc = ia.qz_chunk;
+  auto ia = interp_args<TS, TW, false>(p, L, nullptr, nullptr, nullptr, 1, 1.0);
+  interp_shape<TD>(p, ia, 1, pipe_planes(mz));
+  const int iqc = ia.qz_chunk, giz = (mz + iqc - 1) / iqc;
   const int iparts = std::min(giz, kPipeParts);
   int ic0[kPipeParts + 1];
   for (int k = 0; k <= iparts; ++k) ic0[k] = int((int64_t(k) * giz) / iparts);

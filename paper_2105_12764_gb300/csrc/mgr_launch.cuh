@@ -53,8 +53,6 @@ inline Bufs split_ws(const mgr_plan* p, void* ws) {
   return Bufs{b, b + p->ws_a, b + p->ws_a + p->ws_b};
 }
 
-constexpr int kInterpNW = 8, kInterpRPW = 2;
-
 template <typename TS, typename TW>
 LevelArgs<TS, TW> level_args(const mgr_plan* p, int l) {
   const LevelGeom& g = p->geom[l];
@@ -74,79 +72,81 @@ LevelArgs<TS, TW> level_args(const mgr_plan* p, int l) {
   return a;
 }
 
-// Number of z chunks for `tiles` xy tiles and mz coarse planes: minimise
-// waves x planes streamed per CTA (each chunk also streams ~1.5 halo planes).
-// Chunks may be a single plane: on small levels the plane loop's latency, not
-// the halo's extra work, bounds the pass, so the more CTAs the better.  Chunks
-// are at most max_len planes long (the level pass tabulates its planes).
-inline int choose_chunks(const mgr_plan* p, int64_t tiles, int mz, int ctas_per_sm, int max_len = 1 << 30) {
-  const int64_t slots = int64_t(p->ctx->num_sms) * ctas_per_sm;
-  const int cmin = std::max(1, (mz + max_len - 1) / max_len);
-  int best = cmin;
-  double best_cost = 1e300;
-  const int cmax = std::max(cmin, std::min(mz, 64));
-  for (int c = cmin; c <= cmax; ++c) {
-    const int len = (mz + c - 1) / c;
-    const int cc = (mz + len - 1) / len;
-    const int64_t waves = (tiles * cc + slots - 1) / slots;
-    const double cost = double(waves) * (len + 1.5);
-    if (cost < best_cost - 1e-9) {
-      best_cost = cost;
-      best = c;
-    }
-  }
-  return best;
-}
-
-// Strip height and z chunk length of the level pass (sets a.rows, a.qz_chunk)
-// for `slices` grids of the level at once, `planes` coarse planes of each.  A warp streams rows + 2 units per
-// plane pair (the first and the last in part) over its chunk's planes and about
-// 1.2 more: long strips and chunks repeat least, short ones make more warps.
-// The model: with c warps on an SM a unit takes max(rate, chain / c) cycles of it,
-// `rate` what bounds the pass (FP64: 49 / 32 operations of 16 cycles; FP32: the
-// instructions and the shared-memory and shuffle pipe, measured at 513^3) and
-// `chain` one warp's own latency (measured with few warps).  Warps that are all
-// resident come in whole numbers per SM; more of them than fit run one after
-// another, with half a warp's time lost at the end.  FP32 strips have at most 10
-// rows: longer ones take the L1 cache's share of the memory (513^3: 0.29 ms with
-// 8 or 10 rows, 0.33 with 12 to 14).
-template <int MODE, typename TI, bool QZ, typename TS, typename TW>
-void level_shape(const mgr_plan* p, LevelArgs<TS, TW>& a, int64_t slices = 1, int planes = 1 << 30) {
-  const double rate = sizeof(TS) == 8 ? (MODE == 0 ? 784 : 512) : (MODE == 0 ? 110 : 62);
-  const double chain = sizeof(TS) == 8 ? (MODE == 0 ? 4200 : 2900) : (MODE == 0 ? 1000 : 620);
-  const int max_rows = sizeof(TS) == 8 ? 16 : 10;
-  const int mz = std::min(a.m[0], planes), my = a.m[1], mx = a.m[2];
+// Strip height and z chunk length of the warp-per-strip passes (level pass,
+// interpolation) over my x mz coarse rows and planes.  A warp streams rows +
+// `row_halo` units per plane pair over its chunk's planes and `plane_halo` more:
+// long strips and chunks repeat least, short ones make more warps.  The model:
+// with c warps on an SM a unit takes max(rate, chain / c) cycles of it, `rate` what
+// bounds the pass and `chain` one warp's own latency.  Up to two rounds of resident
+// warps are counted as such, the last one with the warps it has; of more rounds
+// than that, whose warps end one by one, half a warp's time is lost at the end.
+// fixed_rows > 0: only that height.
+struct StripShape {
+  int rows = 1, chunk = 1;
+};
+struct StripModel {
+  double rate, chain, row_halo, plane_halo;
+  int max_rows, fixed_rows;
+};
+template <typename Warps, typename Resident>
+StripShape strip_shape(const mgr_plan* p, int my, int mz, const StripModel& md, Warps warps_of, Resident resident_of) {
   const int64_t sms = p->ctx->num_sms;
+  StripShape out;
   double best = 1e300;
-  for (int rows = 1; rows <= max_rows; ++rows) {
+  for (int rows = 1; rows <= md.max_rows; ++rows) {
     const int strips = (my + rows - 1) / rows;
-    int r = (my + strips - 1) / strips;  // evenly over the strips
-    // FP32 codes: half a 14-row strip, whose places decide a rounding (see level_body)
-    const bool fixed = QZ && MODE == 0 && sizeof(TS) == 4;
-    if (fixed) r = 7;
-    const int64_t warps = level_warps<32>(mx, my, r) * slices;
-    const int64_t resident = std::min<int64_t>(
-        level_ctas<MODE, TS>(),
-        (int64_t(227) << 10) / (level_smem_bytes<MODE, TI, TS, QZ>(r, level_slot_rows(mx, my, r)) + 1024));
+    const int r = md.fixed_rows > 0 ? md.fixed_rows : (my + strips - 1) / strips;  // evenly over the strips
+    const int64_t warps = warps_of(r), resident = resident_of(r);
     // every chunk length that splits the planes evenly, longest first
     for (int len = mz;;) {
       const int chunks = (mz + len - 1) / len;
       const int even = (mz + chunks - 1) / chunks;
       const int64_t w = warps * chunks;
-      const double units = (r + 1.5) * (even + (mz > 1 ? 1.2 : 0.0));
-      const bool all = w <= sms * resident;
-      const double loads = all ? double((w + sms - 1) / sms) : double(w) / sms + 0.5;
-      const double cost = units * loads * std::max(rate, chain / (all ? loads : double(resident)));
+      const double units = (r + md.row_halo) * (even + (mz > 1 ? md.plane_halo : 0.0));
+      const int64_t full = w / (sms * resident), rest = (w - full * sms * resident + sms - 1) / sms;
+      const double round = std::max(md.rate * resident, md.chain);
+      const double cost =
+          units * (full < 2 ? full * round + (rest > 0 ? std::max(md.rate * rest, md.chain) : 0.0)
+                            : (double(w) / sms + 0.5) * round / resident);
       if (cost < best * (1 - 1e-9)) {
         best = cost;
-        a.rows = r;
-        a.qz_chunk = even;
+        out = StripShape{r, even};
       }
       if (even <= 1) break;
       len = even - 1;
     }
-    if (rows >= my || fixed) break;
+    if (rows >= my || md.fixed_rows > 0) break;
   }
+  return out;
+}
+inline int64_t resident_warps(size_t smem, int limit) {
+  return std::min<int64_t>(limit, (int64_t(227) << 10) / int64_t(smem + 1024));
+}
+
+// Shape of the level pass (sets a.rows, a.qz_chunk) for `slices` grids of the level
+// at once, `planes` coarse planes of each.  Rates: FP64 49 / 32 operations of 16
+// cycles; FP32 the instructions and the shared-memory and shuffle pipe, measured
+// at 513^3.  Chains: measured with few warps.  FP32 strips have at most 10 rows:
+// longer ones take the L1 cache's share of the memory (513^3: 0.29 ms with 8 or
+// 10 rows, 0.33 with 12 to 14).  FP32 codes have strips of 7 rows, half of the
+// 14 whose places decide a rounding (see level_body).
+template <int MODE, typename TI, bool QZ, typename TS, typename TW>
+void level_shape(const mgr_plan* p, LevelArgs<TS, TW>& a, int64_t slices = 1, int planes = 1 << 30) {
+  constexpr bool F64 = sizeof(TS) == 8;
+  const StripModel md{F64 ? (MODE == 0 ? 784.0 : 512.0) : (MODE == 0 ? 110.0 : 62.0),
+                      F64 ? (MODE == 0 ? 4200.0 : 2900.0) : (MODE == 0 ? 1000.0 : 620.0),
+                      1.5,
+                      1.2,
+                      F64 ? 16 : 10,
+                      (QZ && MODE == 0 && !F64) ? 7 : 0};
+  const int my = a.m[1], mx = a.m[2];
+  const StripShape s = strip_shape(
+      p, my, std::min(a.m[0], planes), md, [&](int r) { return level_warps<32>(mx, my, r) * slices; },
+      [&](int r) {
+        return resident_warps(level_smem_bytes<MODE, TI, TS, QZ>(r, level_slot_rows(mx, my, r)), level_ctas<MODE, TS>());
+      });
+  a.rows = s.rows;
+  a.qz_chunk = s.chunk;
 }
 
 // Grid of the level pass: warps over the strips, z chunks (sets a.rows, a.qz_chunk;
@@ -193,11 +193,11 @@ template <typename TD, typename TO, typename TS, typename TW, bool PK, bool QZ =
 void launch_interp(const mgr_plan* p, int l, const void* c, const TW* w, void* out, int out_full, cudaStream_t st,
                    double qs = 1.0);
 
-// Arguments of the interpolation of level l (spatial axes) and its (x, y)
-// tile counts; the z chunking is left to the caller.
+// Arguments of the interpolation of level l (spatial axes); its shape is left to
+// the caller.
 template <typename TS, typename TW, bool PK = false>
 InterpArgs<TS, TW> interp_args(const mgr_plan* p, int l, const void* c, const TW* w, void* out, int out_full,
-                               double qs, int* gx, int* gy) {
+                               double qs) {
   const LevelGeom& g = p->geom[l];
   const TS* T = table<TS>(p);
   InterpArgs<TS, TW> a{};
@@ -206,8 +206,7 @@ InterpArgs<TS, TW> interp_args(const mgr_plan* p, int l, const void* c, const TW
     a.m[k] = g.ax[k].m;
     a.s[k] = g.ax[k].s;
     a.N[k] = g.ax[k].N;
-    a.wa[k] = T + g.ax[k].o_wa;
-    a.wb[k] = T + g.ax[k].o_wb;
+    a.slot[k] = T + g.ax[k].o_slot;
   }
   a.c = c;
   a.y_sz = PK ? int64_t(g.ax[1].n) * g.ax[2].n : p->full[1] * p->full[2];
@@ -216,38 +215,52 @@ InterpArgs<TS, TW> interp_args(const mgr_plan* p, int l, const void* c, const TW
   a.c_sz = int64_t(g.ax[1].m) * g.ax[2].m;
   a.c_sy = g.ax[2].m;
   a.out = out;
-  a.out_full = out_full;
   a.qs = qs;
-  a.o_sz = out_full ? a.y_sz : int64_t(g.ax[1].n) * g.ax[2].n;
-  a.o_sy = out_full ? a.y_sy : int64_t(g.ax[2].n);
-  constexpr int BY = kInterpNW * kInterpRPW;
-  *gx = (a.m[2] + 31) / 32;
-  *gy = (a.m[1] + BY - 1) / BY;
+  a.o_sz = out_full ? p->full[1] * p->full[2] : int64_t(g.ax[1].n) * g.ax[2].n;
+  a.o_sy = out_full ? p->full[2] : int64_t(g.ax[2].n);
   return a;
 }
 
-// z chunking of an interpolation launch (sets a.qz_chunk; returns the chunk count)
-template <typename TS, typename TW>
-int interp_chunks(const mgr_plan* p, InterpArgs<TS, TW>& a, int gx, int gy) {
-  const int chunks = choose_chunks(p, int64_t(gx) * gy, a.m[0], 2, kLevelMaxChunk);
-  a.qz_chunk = (a.m[0] + chunks - 1) / chunks;
-  return (a.m[0] + a.qz_chunk - 1) / a.qz_chunk;
+// Shape of an interpolation (sets a.rows, a.qz_chunk) for `slices` grids of the
+// level at once, `planes` coarse planes of each.  Rates: FP64 17 operations of 16
+// cycles; FP32 a unit's 2.2 KB at an SM's share of the HBM.  Strips are short (FP32
+// at most 4 rows, FP64 8): their interpolants take little shared memory, and the
+// L1 cache, through which both columns of a row and the coarse values of
+// neighbouring strips come, keeps the rest (513^3 FP32: 0.22 ms with 4 rows, 0.23
+// with 6, 0.27 with 8; FP64 0.59 with 4 or 8, 0.65 with 10 to 16).
+template <typename TD, typename TS, typename TW>
+void interp_shape(const mgr_plan* p, InterpArgs<TS, TW>& a, int64_t slices = 1, int planes = 1 << 30) {
+  constexpr bool F64 = sizeof(TS) == 8;
+  const StripModel md{F64 ? 270.0 : 102.0, F64 ? 3300.0 : 1050.0, 0.5, 0.4, F64 ? 8 : 4, 0};
+  const int my = a.m[1], mx = a.m[2];
+  const StripShape s = strip_shape(
+      p, my, std::min(a.m[0], planes), md, [&](int r) { return interp_warps(mx, my, r) * slices; },
+      [&](int r) { return resident_warps(interp_smem_bytes<TD, TS, TW>(r, level_slot_rows(mx, my, r)), 16); });
+  a.rows = s.rows;
+  a.qz_chunk = s.chunk;
 }
 
-// z chunks [c0, c1) of the interpolation of level l (c1 < 0: all of them)
+// z chunks [c0, c1) of the interpolation of level l, its shape chosen for `planes`
+// coarse planes at a time (c1 < 0: all of them)
 template <typename TD, typename TO, typename TS, typename TW, bool PK, bool QZ>
 void launch_interp_chunks(const mgr_plan* p, int l, const void* c, const TW* w, void* out, int out_full,
-                          cudaStream_t st, double qs, int c0, int c1) {
-  int gx, gy;
-  InterpArgs<TS, TW> a = interp_args<TS, TW, PK>(p, l, c, w, out, out_full, qs, &gx, &gy);
-  const int gz = interp_chunks(p, a, gx, gy);
+                          cudaStream_t st, double qs, int c0, int c1, int planes = 1 << 30) {
+  InterpArgs<TS, TW> a = interp_args<TS, TW, PK>(p, l, c, w, out, out_full, qs);
+  interp_shape<TD>(p, a, 1, planes);
+  const int gz = (a.m[0] + a.qz_chunk - 1) / a.qz_chunk;
   if (c1 < 0) c1 = gz;
   if (c1 <= c0 || c1 > gz) return;
-  a.bz0 = c0;
-  constexpr size_t sm = interp_smem_bytes<kInterpNW, kInterpRPW, TD, TS, TW>();
-  auto kern = k_interp<kInterpNW, kInterpRPW, TD, TO, TS, TW, PK, QZ>;
+  const size_t sm = interp_smem_bytes<TD, TS, TW>(a.rows, level_slot_rows(a.m[2], a.m[1], a.rows));
+  auto kern = k_interp<TD, TO, TS, TW, true, PK, QZ>;
+  if constexpr (!PK) {
+    if (a.s[2] != 1) kern = k_interp<TD, TO, TS, TW, false, PK, QZ>;
+  }
   raise_smem_limit(kern, sm);
-  kern<<<dim3(gx, gy, c1 - c0), kInterpNW * 32, sm, st>>>(a);
+  // (the grid's y extent is limited to 65535)
+  for (int k = c0; k < c1; k += 65535) {
+    a.bz0 = k;
+    kern<<<dim3(unsigned(interp_warps(a.m[2], a.m[1], a.rows)), unsigned(std::min(c1 - k, 65535))), 32, sm, st>>>(a);
+  }
 }
 
 template <typename TD, typename TO, typename TS, typename TW, bool PK, bool QZ>

@@ -698,62 +698,25 @@ __global__ void __launch_bounds__(32, level_ctas<MODE, TS>()) k_level(const Leve
   level_body<MODE, TI, TD, TS, TW, S1, PK, QZ>(a, blockIdx.x, blockIdx.y + a.bz0, smem_raw);
 }
 
-// CTAs per SM an interpolation CTA of NW warps is compiled for: 16 warps per SM
-// in every configuration, so each thread may use up to 128 registers.
-constexpr int level_ctas_per_sm(int nw) { return nw >= 16 ? 1 : 16 / nw; }
-
-// Plane pairs an interpolation CTA streams at most (its z chunk plus the halo
-// planes before it): the per-plane-pair constants are tabulated once per CTA
-// in shared memory, so the hosts cap the chunk length at kLevelMaxChunk.
-constexpr int kLevelPlanes = 64;
-constexpr int kLevelMaxChunk = kLevelPlanes - 2;
-
-// Copy the element pair (c0, c0+1) of one row into shared memory: one
-// 2-element cp.async when both are in the region, adjacent in memory and
-// aligned (uniform across a warp: every lane of a row has the same parity),
-// else one copy per element.
-template <typename T>
-__device__ __forceinline__ void load_pair(T* dst, const T* src0, const T* src1, bool v0, bool v1, bool contig) {
-  if (v0 && v1 && contig && ((reinterpret_cast<uintptr_t>(src0) & (2 * sizeof(T) - 1)) == 0)) {
-    cp_async(dst, src0, int(2 * sizeof(T)));
-  } else {
-    if (v0) cp_async(dst, src0, int(sizeof(T)));
-    if (v1) cp_async(dst + 1, src1, int(sizeof(T)));
-  }
-}
-
-// Store a pair of output values (to adjacent or separate addresses).  4-byte
-// values are always stored one by one: the warp's stores still coalesce, and
-// the FP32 level pass, bound by instruction issue, saves the alignment test
-// and its branch (measured 7% faster at 513^3).
-template <typename T>
-__device__ __forceinline__ void store_pair(T* p0, T* p1, T a0, T a1, bool w0, bool w1, bool contig) {
-  if constexpr (sizeof(T) == 4) {
-    if (w0) *p0 = a0;
-    if (w1) *p1 = a1;
-    return;
-  }
-  if (w0 && w1 && contig && ((reinterpret_cast<uintptr_t>(p0) & (2 * sizeof(T) - 1)) == 0)) {
-    typename Pair<T>::type v;
-    v.x = a0;
-    v.y = a1;
-    *reinterpret_cast<typename Pair<T>::type*>(p0) = v;
-  } else {
-    if (w0) *p0 = a0;
-    if (w1) *p1 = a1;
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Recomposition interpolation (Sec. II.A, recomposition): level-l values
-// v = c + (P_z x P_y x P_x) v_coarse.  A CTA owns LX x (NW*32/LX*RPW) coarse
-// (x, y) nodes (LX = 32, or 16 in half-warp row groups) and a chunk of
-// coarse z planes; lane l / row k of a row group own the
-// fine block {p(q), p(q)+1} x {p(q), p(q)+1} of their coarse node (the second
-// node only when a fine node lies between q and q+1).  The coarse plane tile
-// (one extra row and column for the right / lower neighbours) is staged in
-// shared memory; the xy interpolants of each coarse plane stay in registers
-// for the fine plane between it and the next one.
+// v = c + (P_z x P_y x P_x) v_coarse, in the level pass's units: one warp takes a
+// strip of coarse rows and a chunk of coarse planes for the coarse x nodes of its
+// lanes, plane pair by plane pair (the coarse plane t and the fine plane before
+// it), each in units of the coarse row qc and the fine row above it.  A lane
+// reads its right neighbour's coarse value itself, so every lane of a warp has
+// outputs, whatever the width (tiles 32 nodes wide took 9 tiles, 288 lanes, for
+// 257 nodes).  The strip's row before the first and the chunk's plane before the
+// first are interpolated only.  The x interpolants of the previous row stay in
+// registers, the xy interpolants of the previous plane in the lane's own
+// shared-memory slots; coefficients and coarse values arrive in a ring of units
+// by asynchronous copies three units ahead.  No step waits for another warp.
+// The output lies at unit stride (the field, or a compact level).
+// What bounds it: FP64 the FP64 pipe (17 operations of 16 cycles a unit), FP32
+// memory (its reads and writes at 0.77 of the copy rate).  513^3, finest level,
+// against 256-thread CTAs over 32 x 16 tiles: FP64 0.721 -> 0.582 ms, FP32 0.219 ->
+// 0.225 ms (the writes of neighbouring warps merge less), 257^3 FP32 0.047 -> 0.039
+// ms, 129^3 FP64 0.036 -> 0.025 ms; 1501 coarse columns of a plane 22 -> 16 us.
 // ---------------------------------------------------------------------------
 template <typename TS, typename TW>
 struct InterpArgs {
@@ -761,287 +724,273 @@ struct InterpArgs {
   int64_t y_sz, y_sy;
   const TW* w;    // coarse values (compact m grid)
   int64_t c_sz, c_sy;
-  void* out;      // level-l values: full grid (out_full) or compact n grid
+  void* out;      // level-l values
   int64_t o_sz, o_sy;
-  int out_full;
   int n[3], m[3];
   int64_t s[3], N[3];
-  const TS* wa[3];
-  const TS* wb[3];
-  int qz_chunk;
-  int bz0;    // first z chunk of this launch (a launch may cover a subset of the chunks)
-  double qs;  // QZ: bin width of the level's class
+  const TS* slot[3];
+  int rows;       // coarse rows per strip
+  int qz_chunk;   // coarse planes per z chunk
+  int bz0;        // first z chunk of this launch (a launch may cover a subset of the chunks)
+  double qs;      // QZ: bin width of the level's class
 };
 
-// Row groups of LX lanes (a warp, or half of one for fields with short coarse
-// rows): a CTA of NW warps owns LX x (NW * 32 / LX * RPW) coarse nodes.
-template <int NW, int RPW, typename TD, typename TW, int LX = 32>
-constexpr size_t interp_table_offset() {
-  constexpr int BY = NW * 32 / LX * RPW, TC = LX == 32 ? 33 : 24;
-  return (sizeof(TD) * 2 * 2 * (2 * BY) * (2 * LX) + sizeof(TW) * 2 * (BY + 1) * TC + 15) / 16 * 16;
+constexpr int kInterpRing = 4;  // units in flight per warp
+// Warps over the coarse nodes of all strips, 32 each.
+__host__ __device__ inline int64_t interp_warps(int mx, int my, int rows) {
+  return (int64_t((my + rows - 1) / rows) * mx + 31) / 32;
 }
-// plane table: per plane pair six offsets (int64), two weights, a flag
-template <int NW, int RPW, typename TD, typename TS, typename TW, int LX = 32>
-constexpr size_t interp_smem_bytes() {
-  return interp_table_offset<NW, RPW, TD, TW, LX>() + kLevelPlanes * (6 * sizeof(int64_t) + 2 * sizeof(TS) + sizeof(int));
+// Shared memory of one warp: the ring (seven coefficients and two coarse values a
+// lane and unit), per unit and lane the four xy interpolants of the last coarse
+// plane, and the y interpolation weights of its rows.
+template <typename TD, typename TS, typename TW>
+__host__ __device__ constexpr size_t interp_smem_bytes(int rows, int slot_rows) {
+  return kInterpRing * 32 * (7 * sizeof(TD) + 2 * sizeof(TW)) +
+         sizeof(TS) * (size_t(rows + 1) * 32 * 4 + size_t(slot_rows) * 2);
 }
 
+// One warp's work: positions 32 bx .. of the strips' nodes and z chunk bz.
 // PK: `c` is the class-packed class of this level (y_sz = n1*n2, y_sy = n2).
 // QZ (with PK): `c` holds int32 codes (TD = int), coefficient = code * qs.
-template <int NW, int RPW, typename TD, typename TO, typename TS, typename TW, bool PK = false, bool QZ = false,
-          int LX = 32>
-__device__ __forceinline__ void interp_body(const InterpArgs<TS, TW>& a, int bx, int by, int bz,
-                                            unsigned char* smem_raw) {
-  static_assert(LX == 32 || LX == 16, "row groups of a warp or half a warp");
-  // coarse tile pitch: LX + 1 columns, padded for half-warp groups so that
-  // the two halves of a warp (RPW rows apart) read different banks
-  constexpr int BY = NW * 32 / LX * RPW, TR = BY + 1, TC = LX == 32 ? 33 : 24, RR = 2 * BY, RC = 2 * LX;
-  using TD2 = typename Pair<TD>::type;
-  TD* stage = reinterpret_cast<TD*>(smem_raw);                                  // [2][2][RR][RC]
-  TW* tile = reinterpret_cast<TW*>(smem_raw + sizeof(TD) * 2 * 2 * RR * RC);  // [2][TR][TC]
-  const int lane = threadIdx.x % LX, warp = threadIdx.x / LX;  // lane in the row group, row group
+// S1: the coefficients lie at unit stride (the finest level, or packed).
+template <typename TD, typename TO, typename TS, typename TW, bool S1, bool PK = false, bool QZ = false>
+__device__ __forceinline__ void interp_body(const InterpArgs<TS, TW>& a, int bx, int bz, unsigned char* smem_raw) {
+  static_assert(S1 || !PK, "a packed class has unit stride");
+  using TS2 = typename Pair<TS>::type;
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr int RING = kInterpRing;
+  const int lid = threadIdx.x & 31;
   const int nz = a.n[0], ny = a.n[1], nx = a.n[2];
   const int mz = a.m[0], my = a.m[1], mx = a.m[2];
-  const int qx0 = bx * LX, qy0 = by * BY;
+  const int rows = a.rows;
+  const int total = ((my + rows - 1) / rows) * mx;
+  const bool out_lane = bx * 32 + lid < total;
+  const int pos = min(bx * 32 + lid, total - 1);
+  const int strip = pos / mx, q = pos - strip * mx;
+  const int qy0 = strip * rows;
+  const int nrow = min(rows, my - qy0);
+  const int units = __reduce_max_sync(FULL, nrow) + 1;
   const int qz0 = bz * a.qz_chunk, qz1 = min(qz0 + a.qz_chunk, mz);
-  const int t_end = min(qz1, mz - 1);
-  const int tcols = min(LX + 1, mx - qx0), trows = min(TR, my - qy0);
+  const int t_start = max(qz0 - 1, 0), t_end = qz1 - 1;
+
   const TD* __restrict__ cin = static_cast<const TD*>(a.c);
   const bool cz = cin == nullptr;  // coefficients of a dropped class: zero
+  TO* __restrict__ out = static_cast<TO*>(a.out);
+  // bounds-checking builds: extents of the buffers; the ITP_* forms check
+  // against them (other builds run the plain accesses)
+#ifdef MGR_DEBUG_BOUNDS
+  const long long n_ci = PK ? (long long)nz * a.y_sz - (long long)mz * a.c_sz : (long long)a.N[0] * a.y_sz;
+  const long long n_w = (long long)mz * a.c_sz;
+  const long long n_o = (long long)nz * a.o_sz;
+#endif
+#define ITP_CP(dst, src)                                                                                           \
+  MGR_GUARD(MGR_PIN(src, cin, n_ci, kDbgInterpC) && MGR_PIN(dst, ring, RING * 7 * 32, kDbgInterpStage), \
+            cp_async(dst, src, int(sizeof(TD))))
+#define ITP_CW(dst, src)                                                                                             \
+  MGR_GUARD(MGR_PIN(src, a.w, n_w, kDbgInterpW) && MGR_PIN(dst, wring, RING * 2 * 32, kDbgInterpStage), \
+            cp_async(dst, src, int(sizeof(TW))))
+#define ITP_O(p, v) MGR_GUARD(MGR_PIN(p, out, n_o, kDbgInterpOut), *(p) = (v))
   const TS qs = QZ ? TS(a.qs) : TS(1);
   // coefficient v plus interpolant b (QZ: code * q + b in one FMA)
   auto cadd = [&](TD v, TS b) -> TS {
     if constexpr (QZ) return fma(code_value<TS>(int(v)), qs, b);
     else return TS(v) + b;
   };
-  TO* __restrict__ out = static_cast<TO*>(a.out);
-  // bounds-checking builds: extents of the buffers; the ITP_* statements
-  // check against them (other builds run the plain statements)
-#ifdef MGR_DEBUG_BOUNDS
-  const long long n_ci = PK ? (long long)nz * a.y_sz - (long long)mz * a.c_sz : (long long)a.N[0] * a.y_sz;
-  const long long n_w = (long long)mz * a.c_sz;
-  const long long n_o = (long long)(a.out_full ? a.N[0] : nz) * a.o_sz;
-  constexpr long long n_stage = 2LL * 2 * RR * RC;
-#endif
-#define ITP_CP(dst, src) \
-  MGR_GUARD(MGR_PIN(src, cin, n_ci, kDbgInterpC) && MGR_PIN(dst, stage, n_stage, kDbgInterpStage), \
-            cp_async(dst, src, int(sizeof(TD))))
-#define ITP_LP(dst, s0, s1, v0, v1, contig)                                                                          \
-  MGR_GUARD((!(v0) || MGR_PIN(s0, cin, n_ci, kDbgInterpC)) && (!(v1) || MGR_PIN(s1, cin, n_ci, kDbgInterpC)) && \
-                MGR_PIN((dst) + 1, stage, n_stage, kDbgInterpStage),                                              \
-            load_pair(dst, s0, s1, v0, v1, contig))
-#define ITP_OP(p0, p1, a0, a1, w0, w1, contig)                                                                          \
-  MGR_GUARD((!(w0) || MGR_PIN(p0, out, n_o, kDbgInterpOut)) && (!(w1) || MGR_PIN(p1, out, n_o, kDbgInterpOut)), \
-            store_pair<TO>(p0, p1, a0, a1, w0, w1, contig))
-
-  // column block of this lane: fine nodes p(qx) and, when a fine node lies
-  // between qx and qx+1, p(qx)+1
-  const int qx = qx0 + lane;
-  const bool ax = qx < mx;
-  const int gx0 = pidx(min(qx, mx - 1), nx);
-  const bool ox1 = ax && qx + 1 < mx && pidx(qx + 1, nx) - gx0 == 2;
-  const TS wax1 = ox1 ? a.wa[2][gx0 + 1] : TS(0), wbx1 = ox1 ? a.wb[2][gx0 + 1] : TS(0);
-  const int gx1 = min(gx0 + 1, nx - 1);
-  const int cc0 = PK ? gx0 : int(fmap(gx0, a.s[2], a.N[2])), cc1 = PK ? gx1 : int(fmap(gx1, a.s[2], a.N[2]));
-  const bool ccontig = cc1 == cc0 + 1;
-  const int pcx1 = gx1 - cidx(gx1);  // packed column of gx1 in a row coarse in y and z
-  const int oc0 = a.out_full ? cc0 : gx0, oc1 = a.out_full ? cc1 : gx1;
-  const bool ocontig = oc1 == oc0 + 1;
-  // row blocks
-  bool ay[RPW], oy1[RPW];
-  TS way1[RPW], wby1[RPW];
-  int cr0[RPW], cr1[RPW], crc0[RPW], crc1[RPW];
-  int64_t or0[RPW], or1[RPW];
-#pragma unroll
-  for (int k = 0; k < RPW; ++k) {
-    const int qy = qy0 + warp * RPW + k;
-    ay[k] = qy < my;
-    const int g0 = pidx(min(qy, my - 1), ny);
-    oy1[k] = ay[k] && qy + 1 < my && pidx(qy + 1, ny) - g0 == 2;
-    way1[k] = oy1[k] ? a.wa[1][g0 + 1] : TS(0);
-    wby1[k] = oy1[k] ? a.wb[1][g0 + 1] : TS(0);
-    const int g1 = min(g0 + 1, ny - 1);
-    cr0[k] = PK ? g0 * nx : int(fmap(g0, a.s[1], a.N[1]) * a.y_sy);
-    cr1[k] = PK ? g1 * nx : int(fmap(g1, a.s[1], a.N[1]) * a.y_sy);
-    // packed rows of a coarse plane
-    crc0[k] = g0 * nx - cidx(g0) * mx;
-    crc1[k] = g1 * nx - cidx(g1) * mx;
-    or0[k] = (a.out_full ? fmap(g0, a.s[1], a.N[1]) : int64_t(g0)) * a.o_sy;
-    or1[k] = (a.out_full ? fmap(g1, a.s[1], a.N[1]) : int64_t(g1)) * a.o_sy;
-  }
-
-  // ---- plane table, computed once by the CTA (instead of by every warp on
-  // every plane pair): entry t - qz0 holds the offsets of plane pair t's
-  // coefficient planes (coarse p(t), and the fine plane before it when there
-  // is one), of its output planes, of the coarse values' plane t, and the
-  // fine plane's z interpolation weights
-  int64_t* itab = reinterpret_cast<int64_t*>(smem_raw + interp_table_offset<NW, RPW, TD, TW, LX>());
-  TS* iwt = reinterpret_cast<TS*>(itab + 6 * kLevelPlanes);
-  int* ifl = reinterpret_cast<int*>(iwt + 2 * kLevelPlanes);
-  auto cplane = [&](int g) -> int64_t {
-    return PK ? int64_t(g) * a.y_sz - int64_t(cidx(g)) * a.c_sz : fmap(g, a.s[0], a.N[0]) * a.y_sz;
+  // coefficient v plus the interpolant between the coarse planes' p and i
+  auto zadd = [&](TD v, TS za, TS p, TS zb, TS i) -> TS {
+    if constexpr (QZ) return cadd(v, za * p + zb * i);
+    else return TS(v) + za * p + zb * i;
   };
-  auto oplane = [&](int g) -> int64_t { return (a.out_full ? fmap(g, a.s[0], a.N[0]) : int64_t(g)) * a.o_sz; };
-  (void)MGR_IN(t_end - qz0, kLevelPlanes, kDbgInterpStage);
-  for (int e = threadIdx.x; e <= t_end - qz0 && e < kLevelPlanes; e += NW * 32) {
-    const int t = qz0 + e, Pc = pidx(t, nz), Pf = Pc - 1;
-    const bool hf = t > qz0 && Pc - pidx(t - 1, nz) == 2;
-    itab[6 * e + 0] = cplane(Pc);
-    itab[6 * e + 1] = hf ? cplane(Pf) : 0;
-    itab[6 * e + 2] = oplane(Pc);
-    itab[6 * e + 3] = oplane(max(Pf, 0));
-    itab[6 * e + 4] = int64_t(t) * a.c_sz;
-    iwt[2 * e + 0] = hf ? a.wa[0][Pf] : TS(0);
-    iwt[2 * e + 1] = hf ? a.wb[0][Pf] : TS(0);
-    ifl[e] = hf ? 1 : 0;
-  }
-  // this thread's copies of the coarse tile: offsets in the coarse plane
-  // (-1: none) and slots
-  constexpr int KT = (TR * TC + NW * 32 - 1) / (NW * 32);
-  int tgo[KT], tso[KT];
-#pragma unroll
-  for (int i = 0; i < KT; ++i) {
-    const int e = threadIdx.x + i * NW * 32;
-    const int r = e / TC, cix = e - r * TC;
-    tgo[i] = (e < trows * TC && cix < tcols) ? int(int64_t(r) * a.c_sy + cix) : -1;
-    tso[i] = r * TC + cix;
-  }
-  const int64_t wtile0 = int64_t(qy0) * a.c_sy + qx0;
-  __syncthreads();  // plane table staged
 
-  // coefficient plane at offset poff of `cin`; zc: a coarse plane
-  auto load_c = [&](TD* sb, int64_t poff, bool zc) {
-    if (cz) return;
-    if constexpr (PK) {
-      const TD* base = cin + poff;
-#pragma unroll
-      for (int k = 0; k < RPW; ++k) {
-        const int r0 = 2 * (warp * RPW + k);
-        if (!ay[k]) continue;
-        if (zc) {
-          // the coarse row g0 of a coarse plane holds its fine column only
-          if (ox1) ITP_CP(sb + r0 * RC + 2 * lane + 1, base + crc0[k] + pcx1);
-          if (oy1[k])
-            ITP_LP(sb + (r0 + 1) * RC + 2 * lane, base + crc1[k] + cc0, base + crc1[k] + cc1, ax, ox1, true);
-        } else {
-          ITP_LP(sb + r0 * RC + 2 * lane, base + cr0[k] + cc0, base + cr0[k] + cc1, ax, ox1, true);
-          if (oy1[k])
-            ITP_LP(sb + (r0 + 1) * RC + 2 * lane, base + cr1[k] + cc0, base + cr1[k] + cc1, ax, ox1, true);
+  // ---- this lane's column (see level_body: slots, swapped pair at the end)
+  const TS wax = a.slot[2][int64_t(kSlot) * q + kSlotWa], wbx = a.slot[2][int64_t(kSlot) * q + kSlotWb];
+  const bool fx = 2 * q + 1 < nx - 1;
+  const bool swp = S1 && 2 * q >= nx - 1;
+  const int ic0 = S1 ? min(2 * q, nx - 2) : int(min(2 * int64_t(q) * a.s[2], a.N[2] - 1));
+  const int64_t icd = S1 ? 1 : (fx ? a.s[2] : 0);
+  const int wcd = q + 1 < mx ? 1 : 0;  // right neighbour's coarse value
+  const int oc0 = min(2 * q, nx - 1);
+  const int rs = S1 ? 1 : int(a.s[1]), rN = S1 ? ny : int(a.N[1]), isy = int(a.y_sy);
+  const int osy = int(a.o_sy), csy = int(a.c_sy);
+  auto cplane = [&](int g) -> int64_t {
+    if (PK) return int64_t(g) * a.y_sz - int64_t(cidx(g)) * a.c_sz;
+    return S1 ? int64_t(g) * a.y_sz : fmap(g, a.s[0], a.N[0]) * a.y_sz;
+  };
+  auto has_fine = [&](int t) { return t > t_start && pidx(t, nz) - pidx(t - 1, nz) == 2; };
+
+  // ---- shared memory: rings, interpolants, y weights
+  TD* ring = reinterpret_cast<TD*>(smem_raw);               // [ring][7][32]: r fine; s, fr, fs own and fine
+  TW* wring = reinterpret_cast<TW*>(ring + RING * 7 * 32);  // [ring][2][32]: own, right neighbour
+  TS* ip_s = reinterpret_cast<TS*>(wring + RING * 2 * 32);  // [units][32][4]
+  TS* ky_s = ip_s + (rows + 1) * 128;                       // [slot rows][2]
+  {
+    // rows qy0 - 2 of the first lane's strip on; rows outside the grid have weights 0
+    const int first_row = __shfl_sync(FULL, qy0, 0) - 2, n = level_slot_rows(mx, my, rows);
+    for (int i = lid; i < n * 2; i += 32) {
+      const int row = first_row + i / 2;
+      ky_s[i] = (row >= 0 && row < my) ? a.slot[1][int64_t(row) * kSlot + kSlotWa + i % 2] : TS(0);
+    }
+    if (cz)
+      for (int i = lid; i < RING * 7 * 32; i += 32) ring[i] = TD(0);
+    __syncwarp();
+    ky_s += (qy0 - 2 - first_row) * 2;  // this lane's unit 0
+  }
+
+  // ---- copies of the next unit (unit lu of plane pair lt)
+  int lt = t_start, lu = 0, lslot = 0;
+  const int lrow0 = 2 * (qy0 - 1) * rs * isy, lrow_max = (rN - 1) * isy;
+  const int wrow0 = (qy0 - 1) * csy, wrow_max = (my - 1) * csy;
+  int lrow = lrow0, wrow = wrow0;
+  bool lhf = false, lc_on = false;
+  const TD *lc = nullptr, *lf = nullptr;
+  const TW* lw = nullptr;
+  auto load_planes = [&]() {
+    const int p = pidx(lt, nz);
+    lhf = !cz && has_fine(lt);
+    lc_on = !cz && lt >= qz0;
+    lw = a.w + (int64_t(lt) * a.c_sz + q);
+    if (!cz) {
+      lc = cin + cplane(p) + ic0;
+      lf = lhf ? cin + cplane(p - 1) + ic0 : lc;
+    }
+  };
+  auto load_unit = [&]() {
+    if (lt <= t_end) {
+      TW* dw = wring + lslot * 64 + lid;
+      const TW* pw = lw + min(max(wrow, 0), wrow_max);
+      ITP_CW(dw, pw);
+      ITP_CW(dw + 32, pw + wcd);
+      if (lu > 0) {
+        TD* dx = ring + lslot * 224 + lid;              // fine column of the coarse row
+        TD* d0 = dx + (swp ? 64 : 32);                  // own columns of the other rows
+        TD* d1 = dx + (swp ? 32 : 64);                  // fine columns
+        const int r = min(max(lrow, 0), lrow_max), s = min(max(lrow - rs * isy, 0), lrow_max);
+        if (lc_on) {
+          if constexpr (PK) {
+            // rows of a coarse plane: the coarse row holds its fine columns only
+            const int qc = min(qy0 - 1 + lu, my - 1);
+            if (fx) ITP_CP(dx, lc - ic0 + (r - qc * mx + q));
+            if (2 * qc - 1 < ny - 1 && qc > 0) {
+              const int o = (2 * qc - 1) * nx - qc * mx;
+              ITP_CP(d0, lc + o);
+              ITP_CP(d1, lc + o + 1);
+            }
+          } else {
+            const TD *pr = lc + r, *ps = lc + s;
+            ITP_CP(dx, swp ? pr : pr + icd);
+            ITP_CP(d0, ps);
+            ITP_CP(d1, ps + icd);
+          }
+        }
+        if (lhf) {
+          const TD *fr = lf + r, *fs = lf + s;
+          ITP_CP(d0 + 64, fr);
+          ITP_CP(d1 + 64, fr + icd);
+          ITP_CP(d0 + 128, fs);
+          ITP_CP(d1 + 128, fs + icd);
         }
       }
-      return;
-    }
-    const TD* base = cin + poff;
-#pragma unroll
-    for (int k = 0; k < RPW; ++k) {
-      const int r0 = 2 * (warp * RPW + k);
-      if (ay[k]) {
-        ITP_LP(sb + r0 * RC + 2 * lane, base + cr0[k] + cc0, base + cr0[k] + cc1, ax, ox1, ccontig);
-        if (oy1[k]) ITP_LP(sb + (r0 + 1) * RC + 2 * lane, base + cr1[k] + cc0, base + cr1[k] + cc1, ax, ox1, ccontig);
+      lslot = (lslot + 1) & (RING - 1);
+      lrow += 2 * rs * isy;
+      wrow += csy;
+      if (++lu == units) {
+        lu = 0;
+        lrow = lrow0;
+        wrow = wrow0;
+        ++lt;
+        if (lt <= t_end) load_planes();
       }
     }
-  };
-  auto issue = [&](int t) {
-    const int e = t - qz0, st = e & 1;
-    TW* tb = tile + st * TR * TC;
-    const TW* src = a.w + itab[6 * e + 4] + wtile0;
-#pragma unroll
-    for (int i = 0; i < KT; ++i)
-      if (tgo[i] >= 0)
-        MGR_GUARD(MGR_PIN(src + tgo[i], a.w, n_w, kDbgInterpW), cp_async(tb + tso[i], src + tgo[i], int(sizeof(TW))));
-    TD* sb = stage + st * 2 * RR * RC;
-    if (t < qz1) load_c(sb, itab[6 * e + 0], true);
-    if (ifl[e]) load_c(sb + RR * RC, itab[6 * e + 1], false);
     cp_commit();
   };
-
-  auto ldc = [&](const TD* p) -> TD2 {
-    TD2 v;
-    if (cz) {
-      v.x = v.y = TD(0);
-    } else {
-      v = *reinterpret_cast<const TD2*>(p);
-    }
-    return v;
-  };
-
-  TS Ip[RPW][4], In[RPW][4];
+  load_planes();
 #pragma unroll
-  for (int k = 0; k < RPW; ++k)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) Ip[k][e] = In[k][e] = TS(0);
+  for (int i = 0; i < RING - 1; ++i) load_unit();
+  int slot = 0;
+  // rows with outputs, by unit: coarse rows u - 1 < nr, the fine rows above them where they exist
+  const unsigned nr = out_lane ? nrow : 0, nrx = fx ? nr : 0;
 
-  issue(qz0);
-  for (int t = qz0; t <= t_end; ++t) {
-    if (t < t_end) {
-      issue(t + 1);
-      cp_wait<1>();
-    } else {
-      cp_wait<0>();
-    }
-    __syncthreads();
-    const int st = (t - qz0) & 1;
-    const TW* tb = tile + st * TR * TC;
-    const TD* sc = stage + st * 2 * RR * RC;
-    const TD* sf = sc + RR * RC;
-    const int te = t - qz0;
-    const bool own_c = t < qz1;
-    const bool hf = ifl[te] != 0;
-    TO* ozc = out + itab[6 * te + 2];
-    TO* ozf = out + itab[6 * te + 3];
-    const TS za = iwt[2 * te + 0], zb = iwt[2 * te + 1];
-#pragma unroll
-    for (int k = 0; k < RPW; ++k) {
-      const int r = warp * RPW + k;
-      const int r0 = 2 * r;
-      const bool act = ax && ay[k];
-      // coarse neighbours (clamped reads stay inside the staged tile)
-      const int rr1 = min(r + 1, trows - 1), cl1 = min(lane + 1, tcols - 1);
-      const int rr0 = min(r, trows - 1), cl0 = min(lane, tcols - 1);
-      const TW w00r = tb[rr0 * TC + cl0];
-      const TS w00 = TS(w00r), w01 = TS(tb[rr0 * TC + cl1]);
-      const TS w10 = TS(tb[rr1 * TC + cl0]), w11 = TS(tb[rr1 * TC + cl1]);
-      In[k][0] = w00;
-      In[k][1] = ox1 ? wax1 * w00 + wbx1 * w01 : TS(0);
-      In[k][2] = oy1[k] ? way1[k] * w00 + wby1[k] * w10 : TS(0);
-      if (ox1 && oy1[k]) {
-        const TS i21 = wax1 * w10 + wbx1 * w11;
-        In[k][3] = way1[k] * In[k][1] + wby1[k] * i21;
+  // ---- one plane pair (HF: with a fine plane)
+  auto plane_pair = [&](auto hf_c, int t) {
+    constexpr bool HF = decltype(hf_c)::value;
+    const int Pc = pidx(t, nz);
+    const bool own_c = t >= qz0;
+    TO* ozc = out + (int64_t(Pc) * a.o_sz + oc0);
+    TO* ozf = out + (int64_t(HF ? Pc - 1 : Pc) * a.o_sz + oc0);
+    const TS* zt = a.slot[0] + int64_t(kSlot) * t;
+    const TS za = HF ? zt[kSlotWa - kSlot] : TS(0), zb = HF ? zt[kSlotWb - kSlot] : TS(0);
+    TS i0p = TS(0), i1p = TS(0);  // x interpolants of coarse row qc-1
+    int qc = qy0 - 1;
+    TS* ip = ip_s + lid * 4;
+    const TS* kp = ky_s;
+    int orow = 2 * qc * osy;
+    const int orow_max = (ny - 1) * osy;
+#pragma unroll 2
+    for (int u = 0; u < units; ++u, ++qc) {
+      // each lane copies, and reads, only its own slots of the rings
+      load_unit();
+      cp_wait<RING - 1>();
+      const TD* d = ring + slot * 224 + lid;
+      const TW* dw = wring + slot * 64 + lid;
+      slot = (slot + 1) & (RING - 1);
+      const TW w0 = dw[0];
+      const TS i0 = TS(w0), i1 = fx ? fma(wbx, TS(dw[32]), wax * i0) : TS(0);
+      const TS2 ky = *reinterpret_cast<const TS2*>(kp);  // interpolation weights of the fine row above
+      kp += 2;
+      const TS i2 = fma(ky.x, i0p, ky.y * i0), i3 = fma(ky.x, i1p, ky.y * i1);
+      TS2 p{}, pp{};
+      if constexpr (HF) {
+        if constexpr (sizeof(TS) == 4) {
+          const float4 v = *reinterpret_cast<const float4*>(ip);
+          p = TS2{v.x, v.y};
+          pp = TS2{v.z, v.w};
+        } else {
+          p = *reinterpret_cast<const TS2*>(ip);
+          pp = *reinterpret_cast<const TS2*>(ip + 2);
+        }
+      }
+      if constexpr (sizeof(TS) == 4) {
+        *reinterpret_cast<float4*>(ip) = make_float4(i0, i1, i2, i3);
       } else {
-        In[k][3] = TS(0);
+        *reinterpret_cast<TS2*>(ip) = TS2{i0, i1};
+        *reinterpret_cast<TS2*>(ip + 2) = TS2{i2, i3};
       }
-      if (act && own_c) {
-        const TD2 c0 = ldc(sc + r0 * RC + 2 * lane);
-        ITP_OP(ozc + or0[k] + oc0, ozc + or0[k] + oc1, TO(w00r), TO(cadd(c0.y, In[k][1])), true, ox1, ocontig);
-        if (oy1[k]) {
-          const TD2 c1 = ldc(sc + (r0 + 1) * RC + 2 * lane);
-          ITP_OP(ozc + or1[k] + oc0, ozc + or1[k] + oc1, TO(cadd(c1.x, In[k][2])), TO(cadd(c1.y, In[k][3])),
-                         true, ox1, ocontig);
-        }
+      ip += 128;
+      i0p = i0;
+      i1p = i1;
+      const bool fine_row = 2 * qc - 1 < ny - 1 && qc > 0;
+      const bool wr = unsigned(u - 1) < nr, wrx = unsigned(u - 1) < nrx;
+      const bool ws = wr && fine_row, wsx = wrx && fine_row;
+      const int oc = min(orow, orow_max), osr = orow - osy;
+      orow += 2 * osy;
+      if (own_c && u > 0) {
+        TO *pr = ozc + oc, *ps = ozc + osr;
+        if (wr) ITP_O(pr, TO(w0));
+        if (wrx) ITP_O(pr + 1, TO(cadd(d[0], i1)));
+        if (ws) ITP_O(ps, TO(cadd(d[32], i2)));
+        if (wsx) ITP_O(ps + 1, TO(cadd(d[64], i3)));
       }
-      if (act && hf) {
-        const TD2 c0 = ldc(sf + r0 * RC + 2 * lane);
-        ITP_OP(ozf + or0[k] + oc0, ozf + or0[k] + oc1, TO(QZ ? cadd(c0.x, za * Ip[k][0] + zb * In[k][0]) : TS(c0.x) + za * Ip[k][0] + zb * In[k][0]),
-                       TO(QZ ? cadd(c0.y, za * Ip[k][1] + zb * In[k][1]) : TS(c0.y) + za * Ip[k][1] + zb * In[k][1]), true, ox1, ocontig);
-        if (oy1[k]) {
-          const TD2 c1 = ldc(sf + (r0 + 1) * RC + 2 * lane);
-          ITP_OP(ozf + or1[k] + oc0, ozf + or1[k] + oc1, TO(QZ ? cadd(c1.x, za * Ip[k][2] + zb * In[k][2]) : TS(c1.x) + za * Ip[k][2] + zb * In[k][2]),
-                         TO(QZ ? cadd(c1.y, za * Ip[k][3] + zb * In[k][3]) : TS(c1.y) + za * Ip[k][3] + zb * In[k][3]), true, ox1, ocontig);
-        }
+      if (HF && u > 0) {
+        TO *pr = ozf + oc, *ps = ozf + osr;
+        if (wr) ITP_O(pr, TO(zadd(d[96], za, p.x, zb, i0)));
+        if (wrx) ITP_O(pr + 1, TO(zadd(d[128], za, p.y, zb, i1)));
+        if (ws) ITP_O(ps, TO(zadd(d[160], za, pp.x, zb, i2)));
+        if (wsx) ITP_O(ps + 1, TO(zadd(d[192], za, pp.y, zb, i3)));
       }
-#pragma unroll
-      for (int e = 0; e < 4; ++e) Ip[k][e] = In[k][e];
     }
-    __syncthreads();  // both stage buffers are reloaded two iterations later
+  };
+  for (int t = t_start; t <= t_end; ++t) {
+    if (has_fine(t)) plane_pair(std::true_type{}, t);
+    else plane_pair(std::false_type{}, t);
   }
 }
 
 #undef ITP_CP
-#undef ITP_LP
-#undef ITP_OP
+#undef ITP_CW
+#undef ITP_O
 
-template <int NW, int RPW, typename TD, typename TO, typename TS, typename TW, bool PK, bool QZ>
-__global__ void __launch_bounds__(NW * 32, level_ctas_per_sm(NW)) k_interp(const InterpArgs<TS, TW> a) {
+template <typename TD, typename TO, typename TS, typename TW, bool S1, bool PK, bool QZ>
+__global__ void __launch_bounds__(32, 16) k_interp(const InterpArgs<TS, TW> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  interp_body<NW, RPW, TD, TO, TS, TW, PK, QZ>(a, blockIdx.x, blockIdx.y, blockIdx.z + a.bz0, smem_raw);
+  interp_body<TD, TO, TS, TW, S1, PK, QZ>(a, blockIdx.x, blockIdx.y + a.bz0, smem_raw);
 }

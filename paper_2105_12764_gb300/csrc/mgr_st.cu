@@ -88,16 +88,16 @@ __global__ void __launch_bounds__(32, level_ctas<MODE, TS>()) k_level_st(const L
   level_body<MODE, TI, TD, TS, TW, S1, false, false, true>(b, blockIdx.x, bz, smem_raw);
 }
 
-template <int NW, int RPW, typename TD, typename TO, typename TS, typename TW>
-__global__ void __launch_bounds__(NW * 32, level_ctas_per_sm(NW)) k_interp_st(const InterpArgs<TS, TW> a, const Slabs sl) {
+template <typename TD, typename TO, typename TS, typename TW, bool S1>
+__global__ void __launch_bounds__(32, 16) k_interp_st(const InterpArgs<TS, TW> a, const Slabs sl) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int j = blockIdx.z / sl.zchunks, bz = blockIdx.z - j * sl.zchunks;
+  const int js = blockIdx.y / sl.zchunks, bz = blockIdx.y - js * sl.zchunks, j = sl.base + js;
   const int t = slab_time(sl, j);
   InterpArgs<TS, TW> b = a;
   b.c = static_cast<const TD*>(a.c) + slab_map(sl, t, 1) * sl.y_ts;
   b.w = a.w + int64_t(j) * sl.w_ts;
   b.out = static_cast<TO*>(a.out) + slab_map(sl, t, sl.out_tfull) * sl.o_ts;
-  interp_body<NW, RPW, TD, TO, TS, TW>(b, blockIdx.x, blockIdx.y, bz, smem_raw);
+  interp_body<TD, TO, TS, TW, S1>(b, blockIdx.x, bz, smem_raw);
 }
 
 // Spatial addressing of one level for the elementwise time passes.
@@ -235,15 +235,20 @@ template <typename TD, typename TO, typename TS, typename TW>
 cudaError_t launch_interp_st(const mgr_plan* p, int l, const TD* c, const TW* w, TO* out, int out_full, Slabs sl,
                              int slabs, cudaStream_t st) {
   if (slabs <= 0) return cudaSuccess;
-  int gx, gy;
-  InterpArgs<TS, TW> a = interp_args<TS, TW>(p, l, c, w, out, out_full, 1.0, &gx, &gy);
-  const int chunks = choose_chunks(p, int64_t(gx) * gy * slabs, a.m[0], 2, kLevelMaxChunk);
-  a.qz_chunk = (a.m[0] + chunks - 1) / chunks;
+  InterpArgs<TS, TW> a = interp_args<TS, TW>(p, l, c, w, out, out_full, 1.0);
+  interp_shape<TD>(p, a, slabs);
   sl.zchunks = (a.m[0] + a.qz_chunk - 1) / a.qz_chunk;
-  constexpr size_t sm = interp_smem_bytes<kInterpNW, kInterpRPW, TD, TS, TW>();
-  auto kern = k_interp_st<kInterpNW, kInterpRPW, TD, TO, TS, TW>;
+  const size_t sm = interp_smem_bytes<TD, TS, TW>(a.rows, level_slot_rows(a.m[2], a.m[1], a.rows));
+  auto kern = a.s[2] == 1 ? k_interp_st<TD, TO, TS, TW, true> : k_interp_st<TD, TO, TS, TW, false>;
   raise_smem_limit(kern, sm);
-  kern<<<dim3(gx, gy, sl.zchunks * slabs), kInterpNW * 32, sm, st>>>(a, sl);
+  // slices in groups: the grid's y extent is limited to 65535
+  const int per = std::max(1, 65535 / sl.zchunks);
+  for (int s0 = 0; s0 < slabs; s0 += per) {
+    Slabs part = sl;
+    part.base = s0;
+    kern<<<dim3(unsigned(interp_warps(a.m[2], a.m[1], a.rows)), sl.zchunks * std::min(per, slabs - s0)), 32, sm, st>>>(
+        a, part);
+  }
   return cudaGetLastError();
 }
 
