@@ -97,7 +97,7 @@ struct SolveDesc {
   TW* w;
   const TW* ta;
   const TW* tb;
-  int64_t lstride, ostride, count, row_pitch;  // count: lines (strided) or rows (contiguous)
+  int64_t lstride, ostride, count;  // count: lines (strided) or rows (contiguous)
   int mline, inner, op, R;
 };
 
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(128) kb_solve_strided(const SolveDesc<TW>* __r
     const SolveDesc<TW> s = d[it.x];
     const int64_t line = int64_t(it.y) * blockDim.x + threadIdx.x;
     if (line < s.count)
-      solve_strided_line<TW, kBatchSolveU<TW>()>(s.f, s.w, s.mline, s.lstride, s.inner, s.ostride, s.ta, s.tb, s.op,
+      solve_strided_line<TW, kBatchSolveU<TW>(), false>(s.f, s.w, s.mline, s.lstride, s.inner, s.ostride, s.ta, s.tb, s.op,
                                                  line,
                              max(int64_t(s.mline) * s.lstride, (s.count / s.inner) * s.ostride));
   }
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(128) kb_solve_contig(const SolveDesc<TW>* __re
   for (int i = blockIdx.x; i < n; i += gridDim.x) {
     const int2 it = items[i];
     const SolveDesc<TW> s = d[it.x];
-    solve_contig_rows<TW>(s.f, s.w, s.mline, s.count, s.row_pitch, s.R, s.ta, s.tb, s.op, int64_t(it.y) * s.R,
+    solve_contig_rows<TW>(s.f, s.w, s.mline, s.count, s.R, s.ta, s.tb, s.op, int64_t(it.y) * s.R,
                           smem_raw);
     __syncthreads();
   }
@@ -475,7 +475,6 @@ struct Builder {
         R = std::max(1, R);
         s.mline = mx;
         s.count = int64_t(mz) * my;
-        s.row_pitch = mx;
         s.R = R;
         csmem = std::max(csmem, solve_contig_smem<TW>(mx, R));
         const int di = int(cdesc.size());

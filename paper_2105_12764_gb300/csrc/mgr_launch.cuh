@@ -292,9 +292,8 @@ cudaError_t launch_x_solve(const mgr_plan* p, TW* f, TW* w, int mx, int64_t line
   }
   if (solve_contig_smem<TW>(mx, 1) > 96 * 1024) {
     // lines too long to stage in shared memory: one thread per line from global memory
-    const int threads = 128;
-    const int blocks = int((lines + threads - 1) / threads);
-    k_solve_strided<TW><<<blocks, threads, 0, st>>>(f, w, mx, 1, 1, lines, mx, ta, tb, op);
+    const int blocks = int((lines + kStridedThreads - 1) / kStridedThreads);
+    k_solve_strided<TW><<<blocks, kStridedThreads, 0, st>>>(f, w, mx, 1, 1, lines, mx, ta, tb, op);
     return cudaGetLastError();
   }
   const int pitch = contig_pitch<TW>(mx);
@@ -305,7 +304,7 @@ cudaError_t launch_x_solve(const mgr_plan* p, TW* f, TW* w, int mx, int64_t line
   const size_t sm = solve_contig_smem<TW>(mx, R);
   const int blocks = int((lines + R - 1) / R);
   raise_smem_limit(k_solve_contig<TW>, sm);
-  k_solve_contig<TW><<<blocks, 128, sm, st>>>(f, w, mx, lines, mx, R, ta, tb, op);
+  k_solve_contig<TW><<<blocks, 128, sm, st>>>(f, w, mx, lines, R, ta, tb, op);
   return cudaGetLastError();
 }
 
@@ -347,18 +346,24 @@ cudaError_t solve_axis_launch(const mgr_plan* p, int l, int axis, TW* f, TW* w, 
     mline = mz; lstride = int64_t(my) * mx; inner = mx; outer = my; ostride = mx;
   }
   const int64_t lines = int64_t(inner) * outer;
-  const size_t ssm = solve_staged_smem<TW>(mline);
   const int64_t staged_below = sizeof(TW) == 4 ? int64_t(MGR_STAGED_LINES_F32) : int64_t(MGR_STAGED_LINES_F64);
-  if (lines < staged_below && ssm <= size_t(100) * 1024 && ssm <= p->ctx->smem_optin) {
-    // few lines (coarse levels): whole lines staged in shared memory, 32 per CTA
-    raise_smem_limit(k_solve_staged<TW>, ssm);
-    k_solve_staged<TW><<<int((lines + kStagedLines - 1) / kStagedLines), 128, ssm, st>>>(f, w, mline, lstride, inner,
-                                                                                       outer, ostride, ta, tb, op);
-    return cudaGetLastError();
+  if (lines < staged_below) {
+    // few lines (coarse levels, planes): whole lines staged in shared memory, fewer
+    // per CTA where there would not be two CTAs per SM, or where they would not fit
+    const int64_t want = 2 * int64_t(p->ctx->num_sms);
+    const size_t limit = std::min<size_t>(size_t(220) * 1024, p->ctx->smem_optin);
+    for (int nl : {32, 16, 8}) {
+      const size_t ssm = solve_staged_smem<TW>(mline, nl);
+      if (ssm > limit || (nl > 8 && lines < want * nl)) continue;
+      auto kern = nl == 32 ? k_solve_staged<TW, 32> : nl == 16 ? k_solve_staged<TW, 16> : k_solve_staged<TW, 8>;
+      raise_smem_limit(kern, ssm);
+      kern<<<unsigned((lines + nl - 1) / nl), kStagedThreads, ssm, st>>>(f, w, mline, lstride, inner, outer, ostride,
+                                                                           ta, tb, op);
+      return cudaGetLastError();
+    }
   }
-  const int threads = 128;
-  const int blocks = int((lines + threads - 1) / threads);
-  k_solve_strided<TW><<<blocks, threads, 0, st>>>(f, w, mline, lstride, inner, outer, ostride, ta, tb, op);
+  const int blocks = int((lines + kStridedThreads - 1) / kStridedThreads);
+  k_solve_strided<TW><<<blocks, kStridedThreads, 0, st>>>(f, w, mline, lstride, inner, outer, ostride, ta, tb, op);
   return cudaGetLastError();
 }
 

@@ -305,8 +305,8 @@ cudaError_t solve_level_st(const mgr_plan* p, int l, TW* f, TW* w, int final_op,
         mline = mt; lstride = Sm; inner = int(Sm); outer = 1; ostride = 0;
       }
       const int64_t lines = int64_t(inner) * outer;
-      k_solve_strided<TW><<<int((lines + 127) / 128), 128, 0, st>>>(f, w, mline, lstride, inner, outer, ostride, ta,
-                                                                    tb, op);
+      k_solve_strided<TW><<<int((lines + kStridedThreads - 1) / kStridedThreads), kStridedThreads, 0, st>>>(
+          f, w, mline, lstride, inner, outer, ostride, ta, tb, op);
     }
     cudaError_t e = cudaGetLastError();
     rec_end(st, name_of(axis), l, double(m) * sizeof(TW) * (op != SOLVE_INPLACE ? 4 : 2),
