@@ -113,40 +113,57 @@ __device__ __forceinline__ int64_t space_full(const SpaceMap& g, int z, int y, i
 
 // D2 (DIR 0) and its inverse (DIR 1) on the slices fine in time, t = 2j + 1
 // between the coarse slices t - 1 and t + 1.  v: level-l values (full grid
-// through the maps when v_full, else compact), c: nodal coefficients.  One
-// warp per (slice, z, y) row.
+// through the maps when v_full, else compact), c: nodal coefficients.  A warp
+// takes 32 consecutive nodes of a slice and runs along time over `per` fine slices:
+// the difference v - c of a coarse slice serves the fine slices on both sides of
+// it, so each coarse slice is read once (four arrays a fine slice instead of six)
+// and takes one operation a node; kTimeAhead slices' loads are in flight.  Bounds:
+// memory, and in FP64 its pipe (three operations a node of a fine slice).
+// 33 x 129^3 FP64: 0.416 -> 0.223 ms.
+constexpr int kTimeAhead = 4;
 template <int DIR, typename TV, typename TC, typename TS>
-__global__ void k_time_fine(TV* v, int v_full, TC* c, SpaceMap g, int nfine, int64_t tS, int64_t tN,
+__global__ void k_time_fine(TV* v, int v_full, TC* c, SpaceMap g, int nfine, int per, int64_t tS, int64_t tN,
                             int64_t space_full_n, const TS* __restrict__ wa, const TS* __restrict__ wb) {
   const int nz = g.n[0], ny = g.n[1], nx = g.n[2];
-  const int64_t rows = int64_t(nfine) * nz * ny;
+  const int64_t Sn = int64_t(nz) * ny * nx, strips = (Sn + 31) / 32;
+  const int64_t tasks = strips * ((nfine + per - 1) / per);
   const int lane = threadIdx.x & 31;
   const int64_t w0 = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5;
   const int64_t nw = (int64_t(gridDim.x) * blockDim.x) >> 5;
-  const int64_t Sn = int64_t(nz) * ny * nx;
-  for (int64_t r = w0; r < rows; r += nw) {
-    const int j = int(r / (int64_t(nz) * ny));
-    const int64_t zy = r - int64_t(j) * nz * ny;
-    const int z = int(zy / ny), y = int(zy - int64_t(z) * ny);
-    const int t = 2 * j + 1;
-    const TS ta = wa[t], tb = wb[t];
-    const int64_t cT0 = fmap(t - 1, tS, tN) * space_full_n, cT = fmap(t, tS, tN) * space_full_n,
-                  cT1 = fmap(t + 1, tS, tN) * space_full_n;
-    const int64_t vT0 = v_full ? cT0 : int64_t(t - 1) * Sn, vT = v_full ? cT : int64_t(t) * Sn,
-                  vT1 = v_full ? cT1 : int64_t(t + 1) * Sn;
-    const bool yz_coarse = is_coarse(z, nz) && is_coarse(y, ny);
-    for (int x = lane; x < nx; x += 32) {
-      const int64_t cs = space_full(g, z, y, x);
-      const int64_t vs = v_full ? cs : (int64_t(z) * ny + y) * nx + x;
-      // coefficients of the coarse slices vanish on their 3D-coarse nodes (the
-      // nodal array holds other levels' values there)
-      const bool cc = yz_coarse && is_coarse(x, nx);
-      const TS c0 = cc ? TS(0) : TS(c[cT0 + cs]), c1 = cc ? TS(0) : TS(c[cT1 + cs]);
-      const TS d = ta * (TS(v[vT0 + vs]) - c0) + tb * (TS(v[vT1 + vs]) - c1);
-      if (DIR == 0) {
-        c[cT + cs] = TC(TS(v[vT + vs]) - d);
-      } else {
-        v[vT + vs] = TV(TS(c[cT + cs]) + d);
+  for (int64_t r = w0; r < tasks; r += nw) {
+    const int part = int(r / strips);
+    const int j0 = part * per, j1 = min(j0 + per, nfine);
+    const int64_t node = (r - part * strips) * 32 + lane;
+    if (node >= Sn) continue;
+    const int zy = int(node / nx), x = int(node - int64_t(zy) * nx);  // (a slice has less than 2^31 nodes)
+    const int z = zy / ny, y = zy - z * ny;
+    const int64_t cs = space_full(g, z, y, x);
+    const int64_t vs = v_full ? cs : node;
+    // coefficients of the coarse slices vanish on their 3D-coarse nodes (the
+    // nodal array holds other levels' values there)
+    const bool cc = is_coarse(z, nz) && is_coarse(y, ny) && is_coarse(x, nx);
+    auto ci = [&](int t) { return fmap(t, tS, tN) * space_full_n + cs; };
+    auto vi = [&](int t) { return v_full ? fmap(t, tS, tN) * space_full_n + vs : int64_t(t) * Sn + vs; };
+    auto coarse = [&](int t) { return TS(v[vi(t)]) - (cc ? TS(0) : TS(c[ci(t)])); };
+    TS e0 = coarse(2 * j0);
+    for (int j = j0; j < j1; j += kTimeAhead) {
+      TS e1[kTimeAhead], own[kTimeAhead];
+#pragma unroll
+      for (int k = 0; k < kTimeAhead; ++k) {
+        if (j + k < j1) {
+          const int t = 2 * (j + k) + 1;
+          e1[k] = coarse(t + 1);
+          own[k] = DIR == 0 ? TS(v[vi(t)]) : TS(c[ci(t)]);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < kTimeAhead; ++k) {
+        if (j + k < j1) {
+          const int t = 2 * (j + k) + 1;
+          if (DIR == 0) c[ci(t)] = TC(own[k] - wa[t] * e0 - wb[t] * e1[k]);
+          else v[vi(t)] = TV(own[k] + wa[t] * e0 + wb[t] * e1[k]);
+          e0 = e1[k];
+        }
       }
     }
   }
@@ -258,9 +275,14 @@ cudaError_t launch_time_fine(const mgr_plan* p, int l, TV* v, int v_full, TC* c,
   const int nfine = g.tax.n - g.tax.m;
   if (nfine <= 0) return cudaSuccess;
   const TS* T = table<TS>(p);
-  const int64_t rows = int64_t(nfine) * g.ax[0].n * g.ax[1].n;
-  const int blocks = int(std::max<int64_t>(1, std::min<int64_t>((rows + 7) / 8, int64_t(p->ctx->num_sms) * 16)));
-  k_time_fine<DIR, TV, TC, TS><<<blocks, 256, 0, st>>>(v, v_full, c, space_map(p, l), nfine, g.tax.s, g.tax.N,
+  // 32 nodes per warp, along all of time unless that leaves SMs without work
+  const int64_t strips = (g.space_fine() + 31) / 32;
+  const int64_t want = int64_t(p->ctx->num_sms) * 48;
+  const int parts = int(std::max<int64_t>(1, std::min<int64_t>(nfine, want / std::max<int64_t>(1, strips))));
+  const int per = (nfine + parts - 1) / parts;
+  const int64_t tasks = strips * ((nfine + per - 1) / per);
+  const int blocks = int(std::max<int64_t>(1, std::min<int64_t>((tasks + 7) / 8, int64_t(p->ctx->num_sms) * 16)));
+  k_time_fine<DIR, TV, TC, TS><<<blocks, 256, 0, st>>>(v, v_full, c, space_map(p, l), nfine, per, g.tax.s, g.tax.N,
                                                         space_full_count(p), T + g.tax.o_wa, T + g.tax.o_wb);
   return cudaGetLastError();
 }
