@@ -523,8 +523,9 @@ cudaError_t host_pipe_t(const mgr_plan* p, const void* host_in, void* host_out, 
 // every coefficient of the coarser levels, and the last plane of an even
 // plane count), then the odd planes in slabs, each slab releasing a part of
 // the finest load-vector pass; the output planes go back as each part of the
-// finest interpolation finishes (part k writes planes [2 qz0, 2 qz1) , the
-// last part up to the last plane).
+// finest interpolation finishes (a part of coarse planes [qz0, qz1) writes the fine
+// plane below each of them: planes 2 qz0 - 1 to 2 qz1 - 2, the last part to the last
+// plane).
 template <typename TD, typename TS, typename TW>
 cudaError_t host_rec_pipe_t(const mgr_plan* p, const void* host_in, void* host_out, const void* dev_in,
                             void* dev_out, void* ws, cudaStream_t st, const PipeCtx& pc, const ForkCtx& fk) {
@@ -580,8 +581,8 @@ cudaError_t host_rec_pipe_t(const mgr_plan* p, const void* host_in, void* host_o
     return e;
   for (int k = 0; k < iparts; ++k) {
     if ((e = cudaStreamWaitEvent(pc.d2h, done_ev[k], 0)) != cudaSuccess) return e;
-    const int z0 = 2 * ic0[k] * iqc;
-    const int z1 = (k == iparts - 1) ? nz : std::min(2 * std::min(ic0[k + 1] * iqc, mz), nz);
+    const int z0 = std::max(2 * ic0[k] * iqc - 1, 0);
+    const int z1 = (k == iparts - 1) ? nz : std::min(2 * ic0[k + 1] * iqc - 1, nz);
     if (z1 > z0 && (e = cudaMemcpyAsync(hout + size_t(z0) * plane, dout + size_t(z0) * plane, size_t(z1 - z0) * plane,
                                         cudaMemcpyDeviceToHost, pc.d2h)) != cudaSuccess)
       return e;
