@@ -326,6 +326,7 @@ cudaError_t recompose_t(const mgr_plan* p, const void* in, void* out, void* ws, 
   Bufs b = split_ws(p, ws);
   auto Fl = [&](int l) { return reinterpret_cast<TW*>(static_cast<char*>(b.F) + p->f_off[l]); };
   // load vector of level l (Sec. II.A.2) from its coefficients, on stream s
+  const bool forked = fk != nullptr && t_recorder == nullptr;
   auto load_vector = [&](int l, cudaStream_t s) -> cudaError_t {
     NvtxRange lv_range("recompose level %d load vector", l);
     const LevelGeom& g = p->geom[l];
@@ -350,7 +351,7 @@ cudaError_t recompose_t(const mgr_plan* p, const void* in, void* out, void* ws, 
         launch_level_chunks<1, TY, TY, TS, TW, PK, QZ>(p, a, rp->c0[k], rp->c0[k + 1], s, pipe_planes(g.ax[0].m));
       }
     } else {
-      launch_level<1, TY, TY, TS, TW, PK, QZ>(p, a, s);
+      launch_level<1, TY, TY, TS, TW, PK, QZ>(p, a, s, forked && sizeof(TS) == 8);
     }
     cudaError_t e = cudaGetLastError();
     const Work wk = work_level_load(p, l, false);
@@ -359,15 +360,21 @@ cudaError_t recompose_t(const mgr_plan* p, const void* in, void* out, void* ws, 
   };
   const int last_lv = std::min(L, ncls - 1);  // levels 1..last_lv have their coefficient class
   const int ls = (PK || QZ) ? 0 : small_levels<TS, TW>(p);  // levels 1..ls run in one CTA
-  const bool fork = fk != nullptr && last_lv > ls && t_recorder == nullptr;
+  const bool fork = forked && last_lv > ls;
   NvtxRange op_range("mgr recompose %s", PK ? (QZ ? "dequantized" : "packed") : "nodal");
   if (rp && cudaStreamWaitEvent(st, rp->even, 0) != cudaSuccess) return cudaGetLastError();
   if (fork) {
     if (cudaEventRecord(fk->ev[0], st) != cudaSuccess || cudaStreamWaitEvent(fk->side, fk->ev[0], 0) != cudaSuccess)
       return cudaGetLastError();
-    // the finest level's pass (most of the work, needed last) on its own
-    // stream from the start, the coarser levels' passes in chain order on the other
-    const bool finest_apart = fk->side2 != nullptr && last_lv == L && L > ls + 1;
+    // The passes in chain order, so that the chain starts at once and the finest
+    // pass fills what it leaves: 257^3 FP64 0.42 ms, against 0.46 with the
+    // finest pass on a stream of its own from the start and 0.51 on one stream;
+    // FP32 0.146, 0.176, 0.183.  Large FP32 fields keep the finest pass apart: it is
+    // bound by memory, and started among the chain's kernels its warps spread
+    // unevenly (500^3 0.60 in order, 0.63 apart; 513^3 0.73, 0.66; 769^3 2.39, 2.11;
+    // 1000 x 700 x 300 1.05, 0.99).
+    const bool finest_apart = fk->side2 != nullptr && last_lv == L && L > ls + 1 && sizeof(TS) == 4 &&
+                              sizeof(TW) == 4 && p->count >= (int64_t(1) << 27);
     if (finest_apart) {
       if (cudaStreamWaitEvent(fk->side2, fk->ev[0], 0) != cudaSuccess) return cudaGetLastError();
       cudaError_t e = load_vector(L, fk->side2);
