@@ -139,8 +139,7 @@ __global__ void __launch_bounds__(128) kb_solve_contig(const SolveDesc<TW>* __re
 }
 
 // The coarse end of every field's hierarchy (its levels of at most a few
-// thousand nodes), one field per CTA: the one-CTA coarse-level bodies of the
-// single-field path, over a list of fields (largest first).
+// thousand nodes), one field per CTA, over a list of fields (largest first).
 #ifndef MGR_BATCH_SMALL_THREADS
 #define MGR_BATCH_SMALL_THREADS 256
 #endif

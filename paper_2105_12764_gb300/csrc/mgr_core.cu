@@ -24,6 +24,7 @@
 // Arithmetic: TS is the stencil type (coefficients, interpolation, K), TW the
 // solve / coarse-workspace type; (double, double) for FP64, (float, float) for
 // FP32, (float, double) for the mixed precision form.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -44,21 +45,7 @@ namespace {
 #include "mgr_solve.cuh"
 #include "mgr_launch.cuh"
 #include "mgr_small.cuh"
-
-// Number of coarse levels (1..ls) the single-CTA kernels take: the largest ls
-// whose level grid (a few thousand nodes) and work arrays fit in shared memory.
-template <typename TS, typename TW>
-int small_levels(const mgr_plan* p) {
-  int ls = 0;
-  for (int l = 1; l <= p->levels && l <= kSmallMaxLevels; ++l) {
-    const LevelGeom& g = p->geom[l];
-    const size_t sm =
-        small_smem_bytes<TS, TW>(g.ax[0].n, g.ax[1].n, g.ax[2].n, g.ax[0].m, g.ax[1].m, g.ax[2].m);
-    if (g.space_fine() > 8192 || sm > size_t(200) * 1024 || sm > p->ctx->smem_optin) break;
-    ls = l;
-  }
-  return ls;
-}
+#include "mgr_cluster.cuh"
 
 template <typename TS, typename TW>
 SmallArgs<TS, TW> small_args(const mgr_plan* p, int ls) {
@@ -90,14 +77,35 @@ SmallArgs<TS, TW> small_args(const mgr_plan* p, int ls) {
   return a;
 }
 
+// Number of coarse levels (1..ls) the one-cluster kernels take: the largest ls whose
+// level grid has at most kClusterNodes nodes and whose slabs fit in shared memory.
+// (Levels up to 40000 nodes there as well: 65^3 FP64 decomposes in 95 us either way and
+// recomposes in 102 instead of 82, where the load passes of the separate launches run
+// beside the chain.)
+constexpr int64_t kClusterNodes = 8192;
+template <typename TS, typename TW>
+int small_levels(const mgr_plan* p) {
+  const int top = std::min(p->levels, kSmallMaxLevels);
+  ClusterArgs<TS, TW> a = cluster_axes(small_args<TS, TW>(p, top));
+  int ls = 0;
+  for (int l = 1; l <= top; ++l) {
+    a.levels = l;
+    const size_t sm = cluster_layout(a);
+    if (p->geom[l].space_fine() > kClusterNodes || sm > size_t(200) * 1024 || sm > p->ctx->smem_optin) break;
+    ls = l;
+  }
+  return ls;
+}
+
 template <typename TD, typename TS, typename TW, bool DEC>
 cudaError_t launch_small(const mgr_plan* p, SmallArgs<TS, TW>& a, cudaStream_t st) {
   const int ls = a.levels;
-  const size_t sm = small_smem_bytes<TS, TW>(a.n[ls][0], a.n[ls][1], a.n[ls][2], a.m[ls][0], a.m[ls][1], a.m[ls][2]);
-  auto kern = DEC ? k_small_dec<TD, TS, TW> : k_small_rec<TD, TS, TW>;
+  ClusterArgs<TS, TW> ca = cluster_axes(a);
+  const size_t sm = cluster_layout(ca);
+  auto kern = DEC ? k_coarse_dec<TD, TS, TW> : k_coarse_rec<TD, TS, TW>;
   raise_smem_limit(kern, sm);
   rec_begin(st);
-  kern<<<1, kSmallThreads, sm, st>>>(a);
+  kern<<<kClusterSize, kClusterThreads, sm, st>>>(ca);
   cudaError_t e = cudaGetLastError();
   double nodes = 0;
   for (int l = 1; l <= ls; ++l) nodes += double(p->geom[l].fine_count());
@@ -205,7 +213,7 @@ cudaError_t decompose_t(const mgr_plan* p, const void* in, void* out, void* ws, 
   Bufs b = split_ws(p, ws);
   TW* F = static_cast<TW*>(b.F);
   TW* cur = nullptr;  // compact level-l values for l < L
-  const int ls = (PK || QZ) ? 0 : small_levels<TS, TW>(p);  // levels ls..1 run in one CTA
+  const int ls = (PK || QZ) ? 0 : small_levels<TS, TW>(p);  // levels ls..1 run in one cluster
   NvtxRange op_range("mgr decompose %s", PK ? (QZ ? "quantized" : "packed") : "nodal");
   for (int l = L; l > ls; --l) {
     NvtxRange level_range("decompose level %d", l);
@@ -270,7 +278,7 @@ cudaError_t decompose_t(const mgr_plan* p, const void* in, void* out, void* ws, 
     cur = nxt;
   }
   if (ls >= 1) {
-    NvtxRange small_range("decompose levels %d..1 in one CTA", ls);
+    NvtxRange small_range("decompose levels %d..1 in one cluster", ls);
     SmallArgs<TS, TW> sa = small_args<TS, TW>(p, ls);
     sa.vin = ls == L ? in : static_cast<const void*>(cur);
     sa.vin_full = ls == L;
@@ -359,7 +367,7 @@ cudaError_t recompose_t(const mgr_plan* p, const void* in, void* out, void* ws, 
     return e;
   };
   const int last_lv = std::min(L, ncls - 1);  // levels 1..last_lv have their coefficient class
-  const int ls = (PK || QZ) ? 0 : small_levels<TS, TW>(p);  // levels 1..ls run in one CTA
+  const int ls = (PK || QZ) ? 0 : small_levels<TS, TW>(p);  // levels 1..ls run in one cluster
   const bool fork = forked && last_lv > ls;
   NvtxRange op_range("mgr recompose %s", PK ? (QZ ? "dequantized" : "packed") : "nodal");
   if (rp && cudaStreamWaitEvent(st, rp->even, 0) != cudaSuccess) return cudaGetLastError();
@@ -390,7 +398,7 @@ cudaError_t recompose_t(const mgr_plan* p, const void* in, void* out, void* ws, 
   // coarsest grid from the nodal positions / class 0
   TW* cur = static_cast<TW*>((L % 2 == 1) ? b.A : b.B);  // level 0 lives where decompose left it
   if (ls >= 1) {
-    // levels 1..ls in one CTA; level ls's values go where the level loop keeps them
+    // levels 1..ls in one cluster; level ls's values go where the level loop keeps them
     TW* lsbuf = (ls % 2 == 1) ? static_cast<TW*>(cur == b.A ? b.B : b.A) : cur;
     SmallArgs<TS, TW> sa = small_args<TS, TW>(p, ls);
     sa.cin = in;

@@ -1,8 +1,8 @@
-// mgr_small.cuh -- the coarse end of the hierarchy in one CTA.
+// mgr_small.cuh -- the coarse end of the hierarchy of one field of a batch in one CTA.
 //
 // Once a level grid fits in shared memory (a few thousand nodes), the tiled
 // level pass, the line solves and the interpolation are each latency-bound
-// launches that use a handful of SMs.  k_small_dec / k_small_rec run all of
+// launches that use a handful of SMs.  small_dec_body / small_rec_body run all of
 // those levels in a single CTA: the level values, coefficients, the
 // intermediate stencil results, the load vector and the coarse values live in
 // shared memory, and every step of Sec. II.A is one parallel loop over its
@@ -17,11 +17,11 @@
 //
 // Stencils use the stencil type TS, solves and coarse values the solve type TW
 // (the same split as the tiled kernels).  Included inside an anonymous
-// namespace after mgr_device.cuh.
+// namespace after mgr_device.cuh.  (A field by itself takes a cluster of CTAs:
+// mgr_cluster.cuh.)
 #pragma once
 
 constexpr int kSmallMaxLevels = 16;
-constexpr int kSmallThreads = 1024;
 
 template <typename TS, typename TW>
 struct SmallArgs {
@@ -62,7 +62,13 @@ constexpr size_t small_smem_bytes(int n0, int n1, int n2, int m0, int m1, int m2
 struct SmallDiv {
   int d;
   float rd;
-  __device__ explicit SmallDiv(int divisor) : d(divisor), rd(1.0f / float(divisor)) {}
+  __device__ explicit SmallDiv(int divisor) : d(divisor) {
+#ifdef __CUDA_ARCH__
+    rd = __frcp_rn(float(divisor));
+#else
+    rd = 1.0f / float(divisor);
+#endif
+  }
   __device__ __forceinline__ int quo(int n) const {
     int q = int(float(n) * rd);
     const int r = n - q * d;
@@ -210,8 +216,8 @@ __device__ __forceinline__ void small_solves(TW* f, const int* m, const int* act
   }
 }
 
-// One field's coarse levels, decomposition: the body of k_small_dec and of
-// the batched one-CTA phase (smem_raw: small_smem_bytes of level a.levels).
+// One field's coarse levels, decomposition: one field of the batched one-CTA
+// phase (smem_raw: small_smem_bytes of level a.levels).
 template <typename TD, typename TS, typename TW>
 __device__ __forceinline__ void small_dec_body(const SmallArgs<TS, TW>& a, unsigned char* smem_raw) {
   const int ls = a.levels;
@@ -280,12 +286,6 @@ __device__ __forceinline__ void small_dec_body(const SmallArgs<TS, TW>& a, unsig
     const int i0 = dc1.quo_rem(dc2.quo_rem(e, i2), i1);
     small_st(out, small_full(a.s0, a.N, i0, i1, i2, a.sz, a.sy), TD(V[e]), a.N, a.sz);
   }
-}
-
-template <typename TD, typename TS, typename TW>
-__global__ void __launch_bounds__(kSmallThreads, 1) k_small_dec(const SmallArgs<TS, TW> a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  small_dec_body<TD, TS, TW>(a, smem_raw);
 }
 
 // One field's coarse levels, recomposition (see small_dec_body).
@@ -358,10 +358,4 @@ __device__ __forceinline__ void small_rec_body(const SmallArgs<TS, TW>& a, unsig
       static_cast<TW*>(a.vout)[e] = V[e];
     }
   }
-}
-
-template <typename TD, typename TS, typename TW>
-__global__ void __launch_bounds__(kSmallThreads, 1) k_small_rec(const SmallArgs<TS, TW> a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  small_rec_body<TD, TS, TW>(a, smem_raw);
 }
