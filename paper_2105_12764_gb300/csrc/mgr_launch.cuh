@@ -80,13 +80,13 @@ LevelArgs<TS, TW> level_args(const mgr_plan* p, int l) {
 // bounds the pass and `chain` one warp's own latency.  Up to two rounds of resident
 // warps are counted as such, the last one with the warps it has; of more rounds
 // than that, whose warps end one by one, half a warp's time is lost at the end.
-// fixed_rows > 0: only that height.
+// tile > 0: only heights that divide it.
 struct StripShape {
   int rows = 1, chunk = 1;
 };
 struct StripModel {
   double rate, chain, row_halo, plane_halo;
-  int max_rows, fixed_rows;
+  int max_rows, tile;
 };
 template <typename Warps, typename Resident>
 StripShape strip_shape(const mgr_plan* p, int my, int mz, const StripModel& md, Warps warps_of, Resident resident_of) {
@@ -94,8 +94,9 @@ StripShape strip_shape(const mgr_plan* p, int my, int mz, const StripModel& md, 
   StripShape out;
   double best = 1e300;
   for (int rows = 1; rows <= md.max_rows; ++rows) {
+    if (md.tile > 0 && md.tile % rows != 0) continue;
     const int strips = (my + rows - 1) / rows;
-    const int r = md.fixed_rows > 0 ? md.fixed_rows : (my + strips - 1) / strips;  // evenly over the strips
+    const int r = md.tile > 0 ? rows : (my + strips - 1) / strips;  // evenly over the strips
     const int64_t warps = warps_of(r), resident = resident_of(r);
     // every chunk length that splits the planes evenly, longest first
     for (int len = mz;;) {
@@ -115,7 +116,7 @@ StripShape strip_shape(const mgr_plan* p, int my, int mz, const StripModel& md, 
       if (even <= 1) break;
       len = even - 1;
     }
-    if (rows >= my || md.fixed_rows > 0) break;
+    if (rows >= my) break;
   }
   return out;
 }
@@ -128,17 +129,18 @@ inline int64_t resident_warps(size_t smem, int limit) {
 // cycles; FP32 the instructions and the shared-memory and shuffle pipe, measured
 // at 513^3.  Chains: measured with few warps.  FP32 strips have at most 10 rows:
 // longer ones take the L1 cache's share of the memory (513^3: 0.29 ms with 8 or
-// 10 rows, 0.33 with 12 to 14).  FP32 codes have strips of 7 rows, half of the
-// 14 whose places decide a rounding (see level_body).
+// 10 rows, 0.33 with 12 to 14).  FP32 codes have strips of 7, 2 or 1 rows, which
+// lie in one of the runs of 14 whose places decide a rounding (see level_body).
 template <int MODE, typename TI, bool QZ, typename TS, typename TW>
 void level_shape(const mgr_plan* p, LevelArgs<TS, TW>& a, int64_t slices = 1, int planes = 1 << 30) {
   constexpr bool F64 = sizeof(TS) == 8;
+  constexpr bool codes = QZ && MODE == 0 && !F64;
   const StripModel md{F64 ? (MODE == 0 ? 784.0 : 512.0) : (MODE == 0 ? 110.0 : 62.0),
                       F64 ? (MODE == 0 ? 4200.0 : 2900.0) : (MODE == 0 ? 1000.0 : 620.0),
                       1.5,
                       1.2,
-                      F64 ? 16 : 10,
-                      (QZ && MODE == 0 && !F64) ? 7 : 0};
+                      F64 ? 16 : codes ? 7 : 10,
+                      codes ? 14 : 0};
   const int my = a.m[1], mx = a.m[2];
   const StripShape s = strip_shape(
       p, my, std::min(a.m[0], planes), md, [&](int r) { return level_warps<32>(mx, my, r) * slices; },
