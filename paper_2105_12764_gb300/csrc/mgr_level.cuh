@@ -579,10 +579,13 @@ __device__ __forceinline__ void level_body(const LevelArgs<TS, TW>& a, int bx, i
         i0p = i0;
         i1p = i1;
       } else {
+        // where the coarse plane has no fine column or fine row, its slots hold
+        // values of coarse nodes, which may be infinite: 0, not only weight 0
+        const bool fine_row = qc > 0 && 2 * qc - 1 < ny - 1;
         r0.c = afine ? cval(vcr.x) : TS(0);
-        r1.c = cval(vcr.y);
-        s0.c = cval(vcs.x);
-        s1.c = cval(vcs.y);
+        r1.c = fx ? cval(vcr.y) : TS(0);
+        s0.c = fine_row ? cval(vcs.x) : TS(0);
+        s1.c = fine_row ? cval(vcs.y) : TS(0);
         if constexpr (HF) {
           r0.f = cval(vfr.x);
           r1.f = cval(vfr.y);

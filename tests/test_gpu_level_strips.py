@@ -86,3 +86,20 @@ def test_fp32_codes_keep_their_values(ctx, shape, prec, crc):
     got = zlib.crc32(codes.cpu().numpy().tobytes())
     plan.close()
     assert got == crc, (shape, prec)
+
+
+@pytest.mark.parametrize("shape", [(33, 33, 33), (40, 37, 66), (34, 36, 130), (150, 171), (9, 33, 17, 18)])
+@pytest.mark.parametrize("dtype", [mgr.MGR_F64, mgr.MGR_F32])
+def test_infinite_coarse_value_stays_in_its_support(ctx, shape, dtype):
+    """An infinite value on a coarse node reaches the nodes that are interpolated from it and no
+    others: it is no coefficient, and the load vector of its level does not see it, at the ends of
+    the axes either."""
+    for at in (0, -1):
+        r = Runner(ctx, shape, None, 1, dtype)
+        c = np.random.default_rng(3).standard_normal(shape)
+        c[(at,) * len(shape)] = np.inf
+        v = r.recompose(c)
+        near = np.zeros(shape, bool)
+        near[tuple(slice(0, 2) if at == 0 else slice(-2 if n % 2 else -1, None) for n in shape)] = True
+        assert np.array_equal(~np.isfinite(v), near), at
+        r.close()
