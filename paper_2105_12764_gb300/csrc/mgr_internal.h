@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "mgr.h"
+#include "mgr_rows.h"
 
 namespace mgr {
 

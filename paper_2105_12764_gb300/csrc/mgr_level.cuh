@@ -358,8 +358,7 @@ __device__ __forceinline__ void level_body(const LevelArgs<TS, TW>& a, int bx, i
   // output columns (MODE 0)
   const int yc0 = PK ? min(2 * q, nx - 1) : int(min(2 * int64_t(q) * a.s[2], a.N[2] - 1));
   const int64_t ycd = S1 ? 1 : a.s[2];
-  // rows: row i of the level sits at min(i * stride, length - 1) * pitch, in
-  // (r) the input and (o) the output
+  // rows of the level (see level_row_offset), in (r) the input and (o) the output
   const int rs = U1 ? 1 : int(a.s[1]), rN = U1 ? ny : int(a.N[1]), isy = int(a.in_sy);
   const int os = S1 ? 1 : int(a.s[1]), oN = S1 ? ny : int(a.N[1]), ysy = int(a.y_sy);
   const int csy = int(a.c_sy);
@@ -396,7 +395,7 @@ __device__ __forceinline__ void level_body(const LevelArgs<TS, TW>& a, int bx, i
   // the fine row above it, in the coarse plane and the fine plane; rows outside
   // the grid read some row of it and carry weight 0
   int lt = t_start, lu = 0, lslot = 0;
-  const int lrow0 = 2 * (qy0 - 1) * rs * isy, lrow_max = (rN - 1) * isy;
+  const int lrow0 = 2 * (qy0 - 1);  // level row of the unit's coarse row
   int lrow = lrow0;
   bool lhf = false;
   const TI *lc = nullptr, *lf = nullptr;
@@ -414,8 +413,8 @@ __device__ __forceinline__ void level_body(const LevelArgs<TS, TW>& a, int bx, i
       TI* d1 = ring1 + lslot * 256;
       TI* dx = ring + lslot * 256 + lid + 32;  // the fine column's slot
       // element offsets of the two rows, clamped into the plane
-      const int r = min(max(lrow, 0), lrow_max), s = min(max(lrow - rs * isy, 0), lrow_max);
-      lrow += 2 * rs * isy;
+      const int r = level_row_offset(lrow, ny, rs, rN, isy), s = level_row_offset(lrow - 1, ny, rs, rN, isy);
+      lrow += 2;
       if constexpr (PK && MODE == 1) {
         // rows of a coarse plane: the coarse row holds its fine columns only
         // (slots without a value: 0, they meet weights 0)
@@ -511,9 +510,6 @@ __device__ __forceinline__ void level_body(const LevelArgs<TS, TW>& a, int bx, i
     TS* ip = ip_s + lid * IPN;
     TS2* ap = reinterpret_cast<TS2*>(acc_s + lid * 2);
     const TS* kp = ky_s;
-    // output rows (element offsets): the coarse row and the fine row above it
-    int orow = 2 * qc * os * ysy;
-    const int orow_max = (oN - 1) * ysy;
 #pragma unroll 2
     for (int u = 0; u < units; ++u, ++qc) {
       // each lane copies, and reads, only its own slots of the ring
@@ -598,10 +594,10 @@ __device__ __forceinline__ void level_body(const LevelArgs<TS, TW>& a, int bx, i
       if constexpr (MODE == 0) {
         const unsigned ur = unsigned(u - 1), us = unsigned(u - 2);
         const bool wr = ur < nr, wrx = ur < nrx, ws = us < ns, wsx = us < nsx;
-        const int oc = min(orow, orow_max), osr = orow - os * ysy;
+        // output rows (element offsets): the coarse row and the fine row above it
+        const int oc = level_row_offset(2 * qc, ny, os, oN, ysy), osr = level_row_offset(2 * qc - 1, ny, os, oN, ysy);
         if (own_c && wr) LVL_W(wp, TW(vcr.x));
         wp += csy;
-        orow += 2 * os * ysy;
         if (wy_c) {
           if constexpr (PK) {
             // rows of a coarse plane leave the coarse nodes out: the coarse row keeps its fine columns
@@ -841,7 +837,7 @@ __device__ __forceinline__ void interp_body(const InterpArgs<TS, TW>& a, int bx,
 
   // ---- copies of the next unit (unit lu of plane pair lt)
   int lt = t_start, lu = 0, lslot = 0;
-  const int lrow0 = 2 * (qy0 - 1) * rs * isy, lrow_max = (rN - 1) * isy;
+  const int lrow0 = 2 * (qy0 - 1);  // level row of the unit's coarse row
   const int wrow0 = (qy0 - 1) * csy, wrow_max = (my - 1) * csy;
   int lrow = lrow0, wrow = wrow0;
   bool lhf = false, lc_on = false;
@@ -867,7 +863,7 @@ __device__ __forceinline__ void interp_body(const InterpArgs<TS, TW>& a, int bx,
         TD* dx = ring + lslot * 224 + lid;              // fine column of the coarse row
         TD* d0 = dx + (swp ? 64 : 32);                  // own columns of the other rows
         TD* d1 = dx + (swp ? 32 : 64);                  // fine columns
-        const int r = min(max(lrow, 0), lrow_max), s = min(max(lrow - rs * isy, 0), lrow_max);
+        const int r = level_row_offset(lrow, ny, rs, rN, isy), s = level_row_offset(lrow - 1, ny, rs, rN, isy);
         if (lc_on) {
           if constexpr (PK) {
             // rows of a coarse plane: the coarse row holds its fine columns only
@@ -894,7 +890,7 @@ __device__ __forceinline__ void interp_body(const InterpArgs<TS, TW>& a, int bx,
         }
       }
       lslot = (lslot + 1) & (RING - 1);
-      lrow += 2 * rs * isy;
+      lrow += 2;
       wrow += csy;
       if (++lu == units) {
         lu = 0;
@@ -926,8 +922,6 @@ __device__ __forceinline__ void interp_body(const InterpArgs<TS, TW>& a, int bx,
     int qc = qy0 - 1;
     TS* ip = ip_s + lid * 4;
     const TS* kp = ky_s;
-    int orow = 2 * qc * osy;
-    const int orow_max = (ny - 1) * osy;
 #pragma unroll 2
     for (int u = 0; u < units; ++u, ++qc) {
       // each lane copies, and reads, only its own slots of the rings
@@ -964,8 +958,7 @@ __device__ __forceinline__ void interp_body(const InterpArgs<TS, TW>& a, int bx,
       const bool fine_row = 2 * qc - 1 < ny - 1 && qc > 0;
       const bool wr = unsigned(u - 1) < nr, wrx = unsigned(u - 1) < nrx;
       const bool ws = wr && fine_row, wsx = wrx && fine_row;
-      const int oc = min(orow, orow_max), osr = orow - osy;
-      orow += 2 * osy;
+      const int oc = level_row_offset(2 * qc, ny, 1, ny, osy), osr = level_row_offset(2 * qc - 1, ny, 1, ny, osy);
       if (own_c && u > 0) {
         TO *pr = ozc + oc, *ps = ozc + osr;
         if (wr) ITP_O(pr, TO(w0));
