@@ -367,6 +367,20 @@ Work slab_work(const mgr_plan* p, int l, bool dec, int slabs, double s_in) {
   return w;
 }
 
+// The same of one pass over the slices fine in time (either direction; s_v: bytes
+// of a level value): they take the values and 3D coefficients of the coarse slices
+// beside them, one operation a node, and read and write one array of their own,
+// two multiply-adds a node.
+Work time_fine_work(const mgr_plan* p, int l, double s_v) {
+  const LevelGeom& g = p->geom[l];
+  const double n = double(g.space_fine()), m = double(g.space_coarse()), sd = double(p->elem);
+  const double fine = double(g.tax.n - g.tax.m), beside = fine > 0 ? fine + 1 : 0;
+  Work w;
+  w.bytes = beside * (n * s_v + (n - m) * sd) + fine * n * (s_v + sd);
+  w.flops = beside * n + fine * n * 4.0;
+  return w;
+}
+
 template <typename TD, typename TS, typename TW>
 cudaError_t decompose_st_t(const mgr_plan* p, const void* in, void* out, void* ws, cudaStream_t st) {
   const int L = p->levels;
@@ -424,8 +438,8 @@ cudaError_t decompose_st_t(const mgr_plan* p, const void* in, void* out, void* w
       e = launch_time_fine<0, TD, TD, TS>(p, l, const_cast<TD*>(static_cast<const TD*>(in)), 1, y, st);
     else
       e = launch_time_fine<0, TW, TD, TS>(p, l, cur, 0, y, st);
-    rec_end(st, "time_coef", l, double(nt - mt) * Sn * (3.0 * (l == L ? sizeof(TD) : sizeof(TW)) + 3.0 * sizeof(TD)),
-            double(nt - mt) * Sn * 6.0);
+    const Work wt = time_fine_work(p, l, double(l == L ? sizeof(TD) : sizeof(TW)));
+    rec_end(st, "time_coef", l, wt.bytes, wt.flops);
     if (e != cudaSuccess) return e;
     // D3: load vectors of the fine-time slices
     {
@@ -529,8 +543,8 @@ cudaError_t recompose_st_t(const mgr_plan* p, const void* in, void* out, void* w
       e = launch_time_fine<1, TD, TD, TS>(p, l, static_cast<TD*>(out), 1, c, st);
     else
       e = launch_time_fine<1, TW, TD, TS>(p, l, nxt, 0, c, st);
-    rec_end(st, "time_interp", l, double(nt - mt) * Sn * (3.0 * (l == L ? sizeof(TD) : sizeof(TW)) + 3.0 * sizeof(TD)),
-            double(nt - mt) * Sn * 6.0);
+    const Work wt = time_fine_work(p, l, double(l == L ? sizeof(TD) : sizeof(TW)));
+    rec_end(st, "time_interp", l, wt.bytes, wt.flops);
     if (e != cudaSuccess) return e;
     cur = nxt;
   }
