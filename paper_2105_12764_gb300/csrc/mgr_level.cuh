@@ -358,7 +358,7 @@ __device__ __forceinline__ void level_body(const LevelArgs<TS, TW>& a, int bx, i
   // output columns (MODE 0)
   const int yc0 = PK ? min(2 * q, nx - 1) : int(min(2 * int64_t(q) * a.s[2], a.N[2] - 1));
   const int64_t ycd = S1 ? 1 : a.s[2];
-  // rows of the level (see level_row_offset), in (r) the input and (o) the output
+  // rows of the level (see StripRows), in (r) the input and (o) the output
   const int rs = U1 ? 1 : int(a.s[1]), rN = U1 ? ny : int(a.N[1]), isy = int(a.in_sy);
   const int os = S1 ? 1 : int(a.s[1]), oN = S1 ? ny : int(a.N[1]), ysy = int(a.y_sy);
   const int csy = int(a.c_sy);
@@ -395,8 +395,7 @@ __device__ __forceinline__ void level_body(const LevelArgs<TS, TW>& a, int bx, i
   // the fine row above it, in the coarse plane and the fine plane; rows outside
   // the grid read some row of it and carry weight 0
   int lt = t_start, lu = 0, lslot = 0;
-  const int lrow0 = 2 * (qy0 - 1);  // level row of the unit's coarse row
-  int lrow = lrow0;
+  StripRows lrow(qy0, rs, rN, isy);
   bool lhf = false;
   const TI *lc = nullptr, *lf = nullptr;
   auto load_planes = [&]() {
@@ -413,13 +412,13 @@ __device__ __forceinline__ void level_body(const LevelArgs<TS, TW>& a, int bx, i
       TI* d1 = ring1 + lslot * 256;
       TI* dx = ring + lslot * 256 + lid + 32;  // the fine column's slot
       // element offsets of the two rows, clamped into the plane
-      const int r = level_row_offset(lrow, ny, rs, rN, isy), s = level_row_offset(lrow - 1, ny, rs, rN, isy);
-      lrow += 2;
+      const int r = lrow.coarse(), s = lrow.fine();
+      lrow.next(lu == 0);
       if constexpr (PK && MODE == 1) {
         // rows of a coarse plane: the coarse row holds its fine columns only
         // (slots without a value: 0, they meet weights 0)
         const int qc = min(max(qy0 - 1 + lu, 0), my - 1);
-        if (fx) LVL_CP(dx, lc - ic0 + (r - qc * mx + q));
+        if (fx && qy0 - 1 + lu == qc) LVL_CP(dx, lc - ic0 + (r - qc * mx + q));
         else *dx = TI(0);
         if (2 * qc - 1 < ny - 1 && qc > 0) {
           const int o = (2 * qc - 1) * nx - qc * mx;
@@ -459,7 +458,7 @@ __device__ __forceinline__ void level_body(const LevelArgs<TS, TW>& a, int bx, i
       lslot = (lslot + 1) & (RING - 1);
       if (++lu == units) {
         lu = 0;
-        lrow = lrow0;
+        lrow.restart();
         ++lt;
         if (lt <= t_end) load_planes();
       }
@@ -510,6 +509,8 @@ __device__ __forceinline__ void level_body(const LevelArgs<TS, TW>& a, int bx, i
     TS* ip = ip_s + lid * IPN;
     TS2* ap = reinterpret_cast<TS2*>(acc_s + lid * 2);
     const TS* kp = ky_s;
+    StripRows orow(qy0, os, oN, ysy);  // output rows
+    orow.rewind();
 #pragma unroll 2
     for (int u = 0; u < units; ++u, ++qc) {
       // each lane copies, and reads, only its own slots of the ring
@@ -594,8 +595,8 @@ __device__ __forceinline__ void level_body(const LevelArgs<TS, TW>& a, int bx, i
       if constexpr (MODE == 0) {
         const unsigned ur = unsigned(u - 1), us = unsigned(u - 2);
         const bool wr = ur < nr, wrx = ur < nrx, ws = us < ns, wsx = us < nsx;
-        // output rows (element offsets): the coarse row and the fine row above it
-        const int oc = level_row_offset(2 * qc, ny, os, oN, ysy), osr = level_row_offset(2 * qc - 1, ny, os, oN, ysy);
+        const int oc = orow.coarse(), osr = orow.above();
+        orow.advance();
         if (own_c && wr) LVL_W(wp, TW(vcr.x));
         wp += csy;
         if (wy_c) {
@@ -837,9 +838,10 @@ __device__ __forceinline__ void interp_body(const InterpArgs<TS, TW>& a, int bx,
 
   // ---- copies of the next unit (unit lu of plane pair lt)
   int lt = t_start, lu = 0, lslot = 0;
-  const int lrow0 = 2 * (qy0 - 1);  // level row of the unit's coarse row
+  StripRows lrow(qy0, rs, rN, isy);
+  lrow.rewind();
   const int wrow0 = (qy0 - 1) * csy, wrow_max = (my - 1) * csy;
-  int lrow = lrow0, wrow = wrow0;
+  int wrow = wrow0;
   bool lhf = false, lc_on = false;
   const TD *lc = nullptr, *lf = nullptr;
   const TW* lw = nullptr;
@@ -863,12 +865,12 @@ __device__ __forceinline__ void interp_body(const InterpArgs<TS, TW>& a, int bx,
         TD* dx = ring + lslot * 224 + lid;              // fine column of the coarse row
         TD* d0 = dx + (swp ? 64 : 32);                  // own columns of the other rows
         TD* d1 = dx + (swp ? 32 : 64);                  // fine columns
-        const int r = level_row_offset(lrow, ny, rs, rN, isy), s = level_row_offset(lrow - 1, ny, rs, rN, isy);
+        const int r = lrow.coarse(), s = lrow.above();
         if (lc_on) {
           if constexpr (PK) {
             // rows of a coarse plane: the coarse row holds its fine columns only
             const int qc = min(qy0 - 1 + lu, my - 1);
-            if (fx) ITP_CP(dx, lc - ic0 + (r - qc * mx + q));
+            if (fx && qy0 - 1 + lu == qc) ITP_CP(dx, lc - ic0 + (r - qc * mx + q));
             if (2 * qc - 1 < ny - 1 && qc > 0) {
               const int o = (2 * qc - 1) * nx - qc * mx;
               ITP_CP(d0, lc + o);
@@ -890,11 +892,11 @@ __device__ __forceinline__ void interp_body(const InterpArgs<TS, TW>& a, int bx,
         }
       }
       lslot = (lslot + 1) & (RING - 1);
-      lrow += 2;
+      lrow.advance();
       wrow += csy;
       if (++lu == units) {
         lu = 0;
-        lrow = lrow0;
+        lrow.rewind();
         wrow = wrow0;
         ++lt;
         if (lt <= t_end) load_planes();
@@ -922,6 +924,8 @@ __device__ __forceinline__ void interp_body(const InterpArgs<TS, TW>& a, int bx,
     int qc = qy0 - 1;
     TS* ip = ip_s + lid * 4;
     const TS* kp = ky_s;
+    StripRows orow(qy0, 1, ny, osy);
+    orow.rewind();
 #pragma unroll 2
     for (int u = 0; u < units; ++u, ++qc) {
       // each lane copies, and reads, only its own slots of the rings
@@ -958,7 +962,8 @@ __device__ __forceinline__ void interp_body(const InterpArgs<TS, TW>& a, int bx,
       const bool fine_row = 2 * qc - 1 < ny - 1 && qc > 0;
       const bool wr = unsigned(u - 1) < nr, wrx = unsigned(u - 1) < nrx;
       const bool ws = wr && fine_row, wsx = wrx && fine_row;
-      const int oc = level_row_offset(2 * qc, ny, 1, ny, osy), osr = level_row_offset(2 * qc - 1, ny, 1, ny, osy);
+      const int oc = orow.coarse(), osr = orow.above();
+      orow.advance();
       if (own_c && u > 0) {
         TO *pr = ozc + oc, *ps = ozc + osr;
         if (wr) ITP_O(pr, TO(w0));

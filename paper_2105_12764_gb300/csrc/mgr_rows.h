@@ -1,5 +1,5 @@
-// mgr_rows.h -- element offset of a row of a level grid within its plane.
-// Plain C++ for host and device.
+// mgr_rows.h -- element offsets of a strip's rows within a plane.  Plain C++ for
+// host and device.
 #pragma once
 
 #ifdef __CUDACC__
@@ -10,16 +10,37 @@
 
 namespace mgr {
 
-// Offset of row i of a level with n rows, s apart on an axis of N rows of `pitch`
-// elements: row i sits at min(i * s, N - 1), rows outside the level are read as its
-// first or last.  The row is clamped before the product with the pitch: a plane has
-// fewer than 2^31 elements, but the last coarse row's i * s may reach nearly 2 N
-// (514 rows of 2097152: row 2 * 2 of the level of 4 rows 256 apart is row 513, and
-// 4 * 256 * 2097152 = 2^31).  i * s itself stays below 2^31 (N <= 2^30).
-MGR_HOST_DEVICE int level_row_offset(int i, int n, int s, int N, int pitch) {
-  const int level_row = i < 0 ? 0 : i < n ? i : n - 1;
-  const int row = level_row * s;
-  return (row < N ? row : N - 1) * pitch;
-}
+// Row i of a level whose rows lie s apart on an axis of N rows of `pitch` elements sits
+// at row min(i * s, N - 1).  Walks the coarse rows i = 2 qc of a strip, and with each the
+// fine row 2 qc - 1 above it, from one before the strip's first.
+//
+// Offsets are unsigned and unclamped until they are used: a plane has fewer than 2^31
+// elements, and a coarse row of the level has i * s < 2 (N - 1), hence an offset below
+// 2^32, where 31 bits would not do (514 rows of 2097152: row 4 of the level of rows 256
+// apart is row 513, and 4 * 256 * 2097152 = 2^31).  Past the end of the axis the offset
+// may wrap; what is returned lies within the plane all the same.
+// (Row indices clamped before a product with the pitch, for every row: the FP32 passes
+// took 1 to 3% longer.)
+struct StripRows {
+  unsigned at, second, half, last;
+  MGR_HOST_DEVICE StripRows(int first, int s, int N, int pitch) {
+    half = unsigned(s) * unsigned(pitch);
+    last = unsigned(N - 1) * unsigned(pitch);
+    second = 2u * unsigned(first) * half;
+    restart();
+  }
+  MGR_HOST_DEVICE int coarse() const { return int(at < last ? at : last); }
+  // Where the row before the axis is read, as row 0.
+  MGR_HOST_DEVICE void restart() { at = second == 0 ? 0u : second - 2u * half; }
+  MGR_HOST_DEVICE void next(bool start) { at = start ? second : at + 2u * half; }  // start: from the first one
+  MGR_HOST_DEVICE int fine() const {
+    const unsigned f = (at > half ? at : half) - half;
+    return int(f < last ? f : last);
+  }
+  // Where only rows of the level are used: before the axis the offset wraps.
+  MGR_HOST_DEVICE void rewind() { at = second - 2u * half; }
+  MGR_HOST_DEVICE void advance() { at += 2u * half; }
+  MGR_HOST_DEVICE int above() const { return int(at - half < last ? at - half : last); }
+};
 
 }  // namespace mgr

@@ -1,10 +1,9 @@
-"""Offsets of a level's rows within a plane, for planes up to the largest the
+"""Offsets of a strip's rows within a plane, for planes up to the largest the
 library takes (fewer than 2^31 elements): level row i sits at full-grid row
-min(i * 2^k, N - 1), so the product of row index and pitch fits in 32 bits only
-once the row is clamped.  The expression the strip kernels use
-(csrc/mgr_rows.h) is compiled for the host and compared with unbounded integers
-over every row a strip may ask for: from the two before the grid to a strip's
-height past its end."""
+min(i * s, N - 1), and i * s * pitch of the last coarse row may reach 2^32.  The walk
+over rows that the strip kernels use (csrc/mgr_rows.h) is compiled for the host and
+compared with unbounded integers: every row of the level is exact, and what a strip
+asks for before the first and past the last row stays within the plane."""
 import ctypes
 import os
 import shutil
@@ -19,29 +18,54 @@ MAX_STRIP = 16
 
 
 @pytest.fixture(scope="module")
-def offset(tmp_path_factory):
+def rows(tmp_path_factory):
     cxx = shutil.which("g++") or shutil.which("c++")
     if cxx is None:
         pytest.skip("no host C++ compiler")
     d = tmp_path_factory.mktemp("rows")
     src, lib = d / "rows.cpp", d / "rows.so"
     src.write_text('#include "mgr_rows.h"\n'
-                   'extern "C" int offset(int i, int n, int s, int N, int pitch) {\n'
-                   '  return mgr::level_row_offset(i, n, s, N, pitch);\n}\n')
+                   'extern "C" void walk(int first, int s, int N, int pitch, int units, int* coarse, int* fine, int* inner,'
+                   ' int* above) {\n'
+                   '  mgr::StripRows r(first, s, N, pitch);\n'
+                   '  for (int pass = 0; pass < 2; ++pass, r.restart())\n'
+                   '    for (int u = 0; u < units; r.next(u == 0), ++u) coarse[u] = r.coarse(), fine[u] = r.fine();\n'
+                   '  for (int pass = 0; pass < 2; ++pass) {\n'
+                   '    r.rewind();\n'
+                   '    for (int u = 0; u < units; r.advance(), ++u) inner[u] = r.coarse(), above[u] = r.above();\n'
+                   '  }\n'
+                   '}\n')
     subprocess.run([cxx, "-std=c++17", "-O2", "-shared", "-fPIC", "-I", CSRC, str(src), "-o", str(lib)], check=True)
-    return ctypes.CDLL(str(lib)).offset
+    walk = ctypes.CDLL(str(lib)).walk
+
+    def rows(first, s, N, pitch, units):
+        out = [(ctypes.c_int * units)() for _ in range(4)]
+        walk(first, s, N, pitch, units, *out)
+        return out
+
+    return rows
 
 
 @pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
-def test_row_offsets(offset, shape):
+def test_row_offsets(rows, shape):
     N, pitch = shape
     assert N * pitch < 2 ** 31
     n, s = N, 1
     while n >= 3:
-        for i in {*range(-2, min(n + 2 * MAX_STRIP, 70)), *range(max(n - 70, -2), n + 2 * MAX_STRIP)}:
-            # compact rows (a level's own values) and full-grid rows
-            assert offset(i, n, 1, n, pitch) == min(max(i, 0), n - 1) * pitch, (n, i)
-            assert offset(i, n, s, N, pitch) == min(max(i, 0) * s, N - 1) * pitch, (n, s, i)
-        n, s = n // 2 + 1, 2 * s
-        if n == 2:
-            break
+        m = n // 2 + 1
+        for first in {*range(min(m, 40)), *range(max(m - 40, 0), m)}:
+            units = MAX_STRIP + 2
+            for step, length in ((1, n), (s, N)):  # a level's own values, the full grid
+                coarse, fine, inner, above = rows(first, step, length, pitch, units)
+                for u in range(units):
+                    qc = first - 1 + u
+                    if qc < m:
+                        at = (2 * max(qc, 0), max(2 * qc - 1, 0))
+                        want = tuple(min(i * step, length - 1) * pitch for i in at)
+                        assert (coarse[u], fine[u]) == want, (n, step, first, u)
+                        if qc >= 0:
+                            assert inner[u] == want[0]
+                        if qc >= 1:
+                            assert above[u] == want[1]
+                    assert all(0 <= v[u] <= (length - 1) * pitch for v in (coarse, fine, inner, above))
+        n, s = m, 2 * s
