@@ -231,10 +231,6 @@ constexpr int kChunks[] = {8, 16, 32, MGR_BATCH_CHUNK_MAX};
 constexpr int kChunks[] = {8, 16, 32};
 #endif
 
-// Resident one-warp level-pass CTAs per SM a persistent launch asks for (the
-// shared memory of 14-row strips allows 18 in FP32).
-constexpr int kLevelResident = 16;
-
 // Coarse rows per interpolation strip, at most (split evenly over a field's strips).
 constexpr int kInterpRows = 4;
 
@@ -322,6 +318,40 @@ struct Builder {
     return cfg_lanes(cand.cfg) == 32 ? level_warps<32>(mx, my, r) : level_warps<16>(mx, my, r);
   }
 
+  // CTAs of `fn` that an SM holds at once: its registers, and the shared memory of
+  // the phase's largest item.  A persistent launch asks for no more (FP64
+  // decomposition strips of 14 rows: 7, FP32: 16).
+  static int resident(const void* fn, int block, size_t smem) {
+    int ctas = 0;
+    if (raise_smem_limit(fn, smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, fn, block, smem) != cudaSuccess)
+      cudaGetLastError();
+    return std::max(ctas, 1);
+  }
+
+  // The level pass's kernel at depth d (depth 0, the finest level, has unit stride).
+  template <int MODE, typename TI>
+  const void* level_fn(int d) const {
+    const bool wide = cfg_lanes(cand.cfg) == 32;
+    if (d == 0)
+      return wide ? reinterpret_cast<const void*>(kb_level<MODE, TI, TD, TS, TW, true>)
+                  : reinterpret_cast<const void*>(kb_level<MODE, TI, TD, TS, TW, true, 16>);
+    return wide ? reinterpret_cast<const void*>(kb_level<MODE, TI, TD, TS, TW, false>)
+                : reinterpret_cast<const void*>(kb_level<MODE, TI, TD, TS, TW, false, 16>);
+  }
+  // Its resident CTAs per SM.
+  template <int MODE, typename TI>
+  int level_resident(int d) const {
+    size_t smem = 0;
+    for (size_t fi = 0; fi < fields.size(); ++fi) {
+      if (!tiled(fi, d)) continue;
+      const LevelGeom& g = fields[fi].p->geom[fields[fi].p->levels - d];
+      const int rows = balanced_chunk(cfg_by(cand.cfg), g.ax[1].m);
+      smem = std::max(smem, level_smem_bytes<MODE, TI, TS>(rows, level_slot_rows(g.ax[2].m, g.ax[1].m, rows)));
+    }
+    return resident(level_fn<MODE, TI>(d), 32, smem);
+  }
+
   // Level-pass phase for all fields at depth d.
   template <int MODE, typename TI>
   void level_phase(int d, bool first_dec) {
@@ -374,16 +404,10 @@ struct Builder {
     ph.desc_off = blob.put(descs.data(), descs.size() * sizeof(descs[0]));
     ph.items_off = blob.put(items.data(), items.size() * sizeof(int4));
     ph.n_items = int(items.size());
-    const bool wide = cfg_lanes(cand.cfg) == 32;
-    if (d == 0)  // the finest level: unit stride
-      ph.fn = wide ? reinterpret_cast<const void*>(kb_level<MODE, TI, TD, TS, TW, true>)
-                   : reinterpret_cast<const void*>(kb_level<MODE, TI, TD, TS, TW, true, 16>);
-    else
-      ph.fn = wide ? reinterpret_cast<const void*>(kb_level<MODE, TI, TD, TS, TW, false>)
-                   : reinterpret_cast<const void*>(kb_level<MODE, TI, TD, TS, TW, false, 16>);
+    ph.fn = level_fn<MODE, TI>(d);
     ph.block = 32;
     ph.smem = smem;
-    ph.grid = std::min(ph.n_items, num_sms * kLevelResident);
+    ph.grid = std::min(ph.n_items, num_sms * resident(ph.fn, ph.block, ph.smem));
     pending.push_back(ph);
   }
 
@@ -440,7 +464,7 @@ struct Builder {
                    : reinterpret_cast<const void*>(kb_interp<TD, TO, TS, TW, false>);
     ph.block = 32;
     ph.smem = smem;
-    ph.grid = std::min(ph.n_items, num_sms * 16);
+    ph.grid = std::min(ph.n_items, num_sms * resident(ph.fn, ph.block, ph.smem));
     pending.push_back(ph);
   }
 
@@ -665,12 +689,13 @@ struct Builder {
   // and the LPT schedule of the items over the persistent CTAs.
   double model_cost(double hbm_bytes_per_us) const {
     double total = 0;
-    const int slots = num_sms * kLevelResident;
     // one warp's time per unit (a row pair of a plane pair), most of the resident warps busy
     const double t_unit_us = sizeof(TS) == 8 ? 4.0 : 0.7;
     int D = 0;
     for (const FieldRef& fr : fields) D = std::max(D, fr.p->levels);
     for (int d = 0; d < D; ++d) {
+      const int slots = num_sms * (op == 1 ? level_resident<1, TD>(d) : d == 0 ? level_resident<0, TD>(d)
+                                                                               : level_resident<0, TW>(d));
       std::vector<double> jobs;
       double bytes = 0;
       for (size_t fi = 0; fi < fields.size(); ++fi) {
