@@ -187,6 +187,11 @@ __device__ __forceinline__ void cluster_st(T* p, int64_t i, T v, int64_t total) 
   if (MGR_IN(i, total, kDbgSmallOut)) p[i] = v;
 }
 
+// Plane `at` of `planes` in the shared memory of CTA `rank` (bounds-checking builds).
+__device__ __forceinline__ bool slab_in(int rank, int at, int planes) {
+  return MGR_IN(rank, kClusterSize, kDbgClusterRank) && MGR_IN(at, planes, kDbgClusterPlane);
+}
+
 // LOCAL: barrier of the CTA, else of the cluster.
 template <bool LOCAL>
 __device__ __forceinline__ void cluster_sync() {
@@ -324,7 +329,9 @@ __device__ __forceinline__ void cluster_correction(const ClusterLevel<TS, TW>& g
         t = t2 + (j - g.i0) * mm;
       } else {  // a neighbour's plane
         const int rr = slab_owner(j == g.n0 - 1 ? g.m0 - 1 : j >> 1, dm0);
-        t = at_rank(t2, rr) + (j - pidx(slab_start(rr, g.m0), g.n0)) * mm;
+        const int plane = j - pidx(slab_start(rr, g.m0), g.n0);
+        if (!slab_in(rr, plane, 2 * slab_planes(g.m0))) continue;
+        t = at_rank(t2, rr) + plane * mm;
       }
       acc += g.k[0][5 * q + o] * t[yx];
     }
@@ -353,6 +360,7 @@ __device__ __forceinline__ void cluster_correction(const ClusterLevel<TS, TW>& g
   for (int e = threadIdx.x; e < ownc * mm; e += kClusterThreads) {
     int yx, k;
     const int q = g.q0 + dmm.quo_rem(e, yx), rr = dper.quo_rem(yx, k);
+    if (!slab_in(rr, q, g.m0)) continue;
     at_rank(fz, rr)[q * per + k] = f[e];
   }
   cluster_sync<false>();
@@ -428,8 +436,9 @@ __device__ __forceinline__ void coarse_dec_level(const ClusterArgs<TS, TW>& a, u
     for (int e = threadIdx.x; e < g.m0 * lines; e += kClusterThreads) {
       int k;
       const int q = dl.quo_rem(e, k), yx = rank * per + k;
-      const int from = slab_owner(q, dm0);
-      const TW v = at_rank(W, from)[(q - slab_start(from, g.m0)) * mm + yx] + fz[q * per + k];
+      const int from = slab_owner(q, dm0), at = q - slab_start(from, g.m0);
+      if (!slab_in(from, at, slab_planes(g.m0))) continue;
+      const TW v = at_rank(W, from)[at * mm + yx] + fz[q * per + k];
       if (l == 1) {
         int x;
         const int y = dm2.quo_rem(yx, x);
@@ -442,7 +451,8 @@ __device__ __forceinline__ void coarse_dec_level(const ClusterArgs<TS, TW>& a, u
         for (int to = 0; to < kClusterSize; ++to) at_rank(V1, to)[q * mm + yx] = v;
       } else {
         const int to = slab_owner(q == g.m0 - 1 ? dk0.d - 1 : q >> 1, dk0);
-        at_rank(V1, to)[(q - pidx(slab_start(to, dk0.d), g.m0)) * mm + yx] = v;
+        const int plane = q - pidx(slab_start(to, dk0.d), g.m0);
+        if (slab_in(to, plane, 2 * slab_planes(dk0.d))) at_rank(V1, to)[plane * mm + yx] = v;
       }
     }
   }
@@ -473,8 +483,8 @@ __device__ __forceinline__ void coarse_rec_level(const ClusterArgs<TS, TW>& a, u
       for (int e = threadIdx.x; e < g.m0 * lines; e += kClusterThreads) {
         int k;
         const int q = dl.quo_rem(e, k), yx = rank * per + k;
-        const int from = slab_owner(q, dm0);
-        at_rank(W, from)[(q - slab_start(from, g.m0)) * mm + yx] -= fz[q * per + k];
+        const int from = slab_owner(q, dm0), at = q - slab_start(from, g.m0);
+        if (slab_in(from, at, slab_planes(g.m0))) at_rank(W, from)[at * mm + yx] -= fz[q * per + k];
       }
     }
   }
@@ -500,12 +510,12 @@ __device__ __forceinline__ void coarse_rec_level(const ClusterArgs<TS, TW>& a, u
       if (LOCAL) {
         if (i0 >= up0 && i0 < up1) W1[(i0 - up0) * n1 * n2 + i12] = v;
       } else {
-        const int to = slab_owner(i0, up);
-        at_rank(W1, to)[(i0 - slab_start(to, up.d)) * n1 * n2 + i12] = v;
+        const int to = slab_owner(i0, up), at = i0 - slab_start(to, up.d);
+        if (slab_in(to, at, slab_planes(up.d))) at_rank(W1, to)[at * n1 * n2 + i12] = v;
       }
     } else if (!LOCAL || (e / 32) % kClusterSize == rank) {
       if (a.vout_full) cluster_st(static_cast<TD*>(a.vout), cluster_full(a, a.s[l], i0, i1, i2), TD(v), a.total);
-      else static_cast<TW*>(a.vout)[i0 * n1 * n2 + i12] = v;
+      else cluster_st(static_cast<TW*>(a.vout), i0 * n1 * n2 + i12, v, g.n0 * n1 * n2);
     }
   }
   __syncthreads();
@@ -545,7 +555,7 @@ __global__ void __cluster_dims__(kClusterSize, 1, 1) __launch_bounds__(kClusterT
         const int i0 = g.i0 + dn1.quo_rem(dn2.quo_rem(e, i2), i1);
         V[e] = TW(cluster_ld(static_cast<const TD*>(a.vin), cluster_full(a, a.s[ls], i0, i1, i2), a.total));
       } else {
-        V[e] = static_cast<const TW*>(a.vin)[first + e];
+        V[e] = cluster_ld(static_cast<const TW*>(a.vin), first + e, g.n0 * g.n1 * g.n2);
       }
     }
   }

@@ -6,11 +6,6 @@
 __device__ __forceinline__ int pidx(int q, int n) { return min(2 * q, n - 1); }
 __device__ __forceinline__ bool is_coarse(int i, int n) { return ((i & 1) == 0) || (i == n - 1); }
 __device__ __forceinline__ int cidx(int i) { return (i + 1) >> 1; }
-// first fine node of the stencil region of coarse node q0, moved down to a coarse node
-__device__ __forceinline__ int region_start(int q0, int n) {
-  const int r = pidx(q0, n) - 2;
-  return (r & 1) ? r - 1 : r;
-}
 __device__ __forceinline__ int64_t fmap(int i, int64_t s, int64_t N) {
   int64_t f = int64_t(i) * s;
   return f < N - 1 ? f : N - 1;

@@ -181,10 +181,10 @@ struct DebugRecord {
   long long extent;
 };
 enum : int {
-  kDbgLevelIn = 1, kDbgLevelY = 2, kDbgLevelW = 3, kDbgLevelF = 4, kDbgLevelStage = 5, kDbgLevelTile = 6,
+  kDbgLevelIn = 1, kDbgLevelY = 2, kDbgLevelW = 3, kDbgLevelF = 4, kDbgLevelStage = 5,
   kDbgInterpC = 11, kDbgInterpW = 12, kDbgInterpOut = 13, kDbgInterpStage = 14,
   kDbgSolveF = 21, kDbgSolveW = 22, kDbgSolveSmem = 23,
-  kDbgSmallIn = 31, kDbgSmallOut = 32, kDbgCoarsestY = 41, kDbgCoarsestW = 42,
+  kDbgSmallIn = 31, kDbgSmallOut = 32, kDbgClusterRank = 33, kDbgClusterPlane = 34, kDbgCoarsestY = 41, kDbgCoarsestW = 42,
 };
 // Read and clear the records of every translation unit (bounds-checking
 // builds; others report nothing): returns the number of violations since the
