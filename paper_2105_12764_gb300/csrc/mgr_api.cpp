@@ -157,7 +157,7 @@ bool packed_op(int op) { return (op & 0xff) >= OP_DEC_PACKED; }
 // The side streams and events of a forked recomposition graph (graph_mu held).
 bool ensure_fork(mgr_plan* p) {
   if (p->side) return true;
-  if (!p->side2 && cudaStreamCreateWithFlags(&p->side2, cudaStreamNonBlocking) != cudaSuccess) return false;
+  if (mgr::finest_apart(p) && !p->side2 && cudaStreamCreateWithFlags(&p->side2, cudaStreamNonBlocking) != cudaSuccess) return false;
   if (cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking) != cudaSuccess) return false;
   p->fork_ev.assign(p->levels + 1, nullptr);
   for (auto& e : p->fork_ev)

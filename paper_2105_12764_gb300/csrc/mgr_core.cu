@@ -295,9 +295,9 @@ cudaError_t decompose_t(const mgr_plan* p, const void* in, void* out, void* ws, 
 // interpolation only.  PK: `in` is class-packed (its first class_off[ncls]
 // elements are read) and must not overlap `out`.
 // QZ (with PK): `in` holds int32 codes with the bin widths bins[0..L].
-// fk (graph capture only): the load-vector passes of all levels run on
-// fk->side (the finest level's on fk->side2) ahead of the solve /
-// interpolation chain on st, each level into its own load-vector buffer; st
+// fk (graph capture only): the load-vector passes of all levels run on fk->side,
+// coarsest first, ahead of the solve / interpolation chain on st (the finest one
+// on fk->side2 where finest_apart), each level into its own load-vector buffer; st
 // waits for level l's before its solves.
 // The recomposition of a pipelined host-buffer call: every pass waits for
 // `even` (the planes holding the coefficients of the coarser levels are on the
@@ -377,19 +377,15 @@ cudaError_t recompose_t(const mgr_plan* p, const void* in, void* out, void* ws, 
     // The passes in chain order, so that the chain starts at once and the finest
     // pass fills what it leaves: 257^3 FP64 0.42 ms, against 0.46 with the
     // finest pass on a stream of its own from the start and 0.51 on one stream;
-    // FP32 0.146, 0.176, 0.183.  Large FP32 fields keep the finest pass apart: it is
-    // bound by memory, and started among the chain's kernels its warps spread
-    // unevenly (500^3 0.60 in order, 0.63 apart; 513^3 0.73, 0.66; 769^3 2.39, 2.11;
-    // 1000 x 700 x 300 1.05, 0.99).
-    const bool finest_apart = fk->side2 != nullptr && last_lv == L && L > ls + 1 && sizeof(TS) == 4 &&
-                              sizeof(TW) == 4 && p->count >= (int64_t(1) << 27);
-    if (finest_apart) {
+    // FP32 0.146, 0.176, 0.183.
+    const bool apart = fk->side2 != nullptr && last_lv == L && L > ls + 1 && finest_apart(p);
+    if (apart) {
       if (cudaStreamWaitEvent(fk->side2, fk->ev[0], 0) != cudaSuccess) return cudaGetLastError();
       cudaError_t e = load_vector(L, fk->side2);
       if (e != cudaSuccess) return e;
       if ((e = cudaEventRecord(fk->ev[L], fk->side2)) != cudaSuccess) return e;
     }
-    for (int l = ls + 1; l <= (finest_apart ? L - 1 : last_lv); ++l) {
+    for (int l = ls + 1; l <= (apart ? L - 1 : last_lv); ++l) {
       cudaError_t e = load_vector(l, fk->side);
       if (e != cudaSuccess) return e;
       if ((e = cudaEventRecord(fk->ev[l], fk->side)) != cudaSuccess) return e;
@@ -607,6 +603,13 @@ cudaError_t host_rec_pipe_t(const mgr_plan* p, const void* host_in, void* host_o
 }
 
 }  // namespace
+
+// FP32 fields from 2^27 nodes on.  Apart against in order: nodal 257^3 1.07, 385^3
+// 1.05, 449^3 to 511^3 1.01, 512^3 to 520^3 0.99, 560^3 1.00, 640^3 1.01, and 0.98 to
+// 1.04 over six ragged fields of 1.2e8 to 2.1e8 nodes; packed 257^3 1.01, 385^3 0.99,
+// 449^3 to 560^3 0.95 to 0.98, 640^3 0.99, ragged 0.93 to 1.00.  So the line is not sharp: it
+// keeps the small fields, where apart loses, and the large packed ones, where it gains.
+bool finest_apart(const mgr_plan* p) { return p->form == kFormF32 && p->count >= (int64_t(1) << 27); }
 
 cudaError_t enqueue_recompose_host_pipe(const mgr_plan* p, const void* host_in, void* host_out, const void* dev_in,
                                         void* dev_out, void* ws, cudaStream_t st, const PipeCtx& pc,

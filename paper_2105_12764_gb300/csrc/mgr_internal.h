@@ -104,8 +104,8 @@ struct mgr_plan {
   // workspace layout (bytes)
   size_t ws_a = 0, ws_b = 0, ws_f = 0, ws_g = 0, ws_bytes = 0;  // ws_g: 4D time-slice load vectors
   std::vector<size_t> f_off;  // byte offset of level l's load vector in the F region (l = 1..L)
-  // side stream and events of the forked recomposition graph (created on the
-  // first capture, under graph_mu)
+  // side streams and events of the forked recomposition graph (created on the
+  // first capture, under graph_mu; side2 where finest_apart)
   cudaStream_t side = nullptr, side2 = nullptr;
   std::vector<cudaEvent_t> fork_ev;
   // copy streams and events of the pipelined host-buffer decomposition
@@ -242,8 +242,11 @@ cudaError_t enqueue_recompose_st(const mgr_plan* p, const void* in, void* out, v
 struct ForkCtx {
   cudaStream_t side;
   cudaEvent_t* ev;
-  cudaStream_t side2;  // the finest level's pass (may be null: everything on side)
+  cudaStream_t side2;  // the finest level's pass where finest_apart (may be null: everything on side)
 };
+// whether the plan's recompositions run the finest level's load-vector pass on a
+// stream of its own
+bool finest_apart(const mgr_plan* p);
 cudaError_t enqueue_recompose_fork(const mgr_plan* p, int op, const void* in, int ncls, const double* bins, void* out,
                                    void* ws, cudaStream_t st, const ForkCtx& fk);
 // Decomposition with pinned host buffers, pipelined (graph capture only): the
