@@ -37,8 +37,9 @@
 //
 // What bounds it.  FP64: the FP64 pipe, one SM-wide operation per 16 cycles and
 // warp; a unit takes 49 of them in decomposition, 32 in recomposition (level_shape
-// counts with that).  FP32: no single unit (at 513^3 issue slots 50%, shared-memory
-// and shuffle pipe 62%, DRAM 48%), but the dependent chains of about 12 warps per
+// counts with that); busy 91% of the finest pass at 257^3.  FP32: no single unit
+// (385^3, finest level: issue slots 43%, shared-memory and shuffle pipe 67%, DRAM
+// 52%), but the dependent chains of about 11 warps per
 // SM.  513^3, finest level, against the earlier pass of 8-warp tiles with two CTA
 // barriers per plane pair: FP64 decomposition 2.12 -> 1.82 ms, recomposition 1.48
 // -> 1.12 ms; FP32 0.375 -> 0.303 and 0.248 -> 0.174 ms.  65^3 FP64, where the
